@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_cell_fx(FxArgs a) {
     }
     const double dg = (a.diag + 0.5 * q2) * a.dt;
     bound += fabs(dg);
-    s_cbad = !(bound < 4.1);
+    s_cbad = !(bound < 4.1) || fabs(dg) >= 3.0;     // (with |dt V| < 1 a digit holds the sum)
     s_diag = digits28(s_cbad ? 0 : __double2ll_rn(dg * 144115188075855872.0));
     if (OBS) {
       const double* Ao = a.Ap_obs_cell ? a.Ap_obs_cell + 3 * cell : a.Ap_obs;
