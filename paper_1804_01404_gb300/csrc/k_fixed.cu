@@ -591,10 +591,14 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_cell_fx(FxArgs a) {
     const ll X = join31(u.x, u.y), Y = join31(u.z, u.w);
     if (out) out[pg] = make_double2(to_double(X, s), to_double(Y, s));
     if (rho) {
-      const int2 ux = digits27<6>(X), uy = digits27<6>(Y);
+      // |u|^2 2^2k from the values shifted up by their leading zeros, so that small values keep their digits
+      // (LDA takes the cube root of the density)
+      const int k2 = __clzll((X ^ (X >> 63)) | (Y ^ (Y >> 63))) - 4;
+      const int2 ux = digits27<6>(X << k2), uy = digits27<6>(Y << k2);
       const ll P = mw(ux.x, ux.x, mw(uy.x, uy.x, 0)), Q = mw(ux.x, ux.y, mw(uy.x, uy.y, 1LL << 18));
       const ll R = mw(ux.y, ux.y, mw(uy.y, uy.y, 1LL << 46));
-      atomicAdd(rho + pg, __ll2double_rn((P << 7) + (Q >> 19) + (R >> 47)) * rfac);
+      const double d = __ll2double_rn((P << 7) + (Q >> 19) + (R >> 47));
+      if (d != 0.0) atomicAdd(rho + pg, __hiloint2double(__double2hiint(d) - 2 * k2 * (1 << 20), __double2loint(d)) * rfac);
     }
     if (OBS == 1) {
       const int2 ux = digits27<8>(X), uy = digits27<8>(Y);

@@ -1,5 +1,5 @@
 """Where the fixed-point Taylor launches of FP64 orbitals could fall short of FP64: the digits of the diagonal
-coefficient."""
+coefficient and the density of points far below an orbital's largest value."""
 import numpy as np
 import pytest
 
@@ -12,6 +12,23 @@ from paper_1804_01404_gb300 import tdks, workloads as W  # noqa: E402
 def box(n, h, periodic, norb, atoms=(), proj=None):
     return W.System(n=n, h=h, periodic=periodic, atoms=list(atoms), proj=proj or W.Projectors(r_cut=1.5),
                     kpts=np.zeros((1, 3)), kw=np.ones(1), norb=norb, dt=0.02, field=W.Field("none"))
+
+
+@pytest.mark.parametrize("n,periodic", [((19, 10, 12), False), ((16, 16, 16), True), ((9, 13, 20), False)], ids=str)
+def test_density_of_small_values(n, periodic):
+    """Every point of the density to FP64 accuracy: 2^-53 from the orbitals' rounding in each of the squares, as
+    much from the digits of the product, and an addition per orbital, below 2e-15 for eight of them."""
+    s = box(n, (0.45, 0.5, 0.4), periodic, 8)
+    ctx = tdks.Context(s, precision="f64")
+    u0 = W.initial_orbitals(s, 4)
+    u0[0, :, 3, 4:6, :] *= 1e-9                          # values of 1e-9 of an orbital's largest beside ordinary ones
+    u = torch.from_numpy(u0).cuda()
+    ctx.update_potential(u)
+    ctx.step(u, 0.0, 1e-7)
+    rho, v = ctx.grid_array(2).cpu().numpy(), u.cpu().numpy()
+    ref = 2 * (v.real ** 2 + v.imag ** 2).sum((0, 1))
+    assert ref.min() < 1e-9 * ref.max()
+    assert np.abs(rho / ref - 1).max() < 2e-15
 
 
 def test_diagonal_beyond_its_digits():
