@@ -24,8 +24,8 @@
 // every other) and after the nonlocal scatter.
 //
 // Ranges: |X| < 2^60 after every stage, checked at every point; an orbital that leaves it (an unstable
-// step), holds a non-finite value, or meets a potential or a wave vector outside the range of the
-// coefficients writes nothing but its flag, and the FP64 kernel propagates it (launched after this one;
+// step), holds a non-finite value, decays into a vacuum (kFxRange), or meets a potential or a wave vector outside
+// the range of the coefficients writes nothing but its flag, and the FP64 kernel propagates it (launched after this one;
 // its CTAs return at once for the others: 3 us for 8 orbitals, 6 us for 1024).
 #include <cuda_runtime.h>
 
@@ -42,6 +42,11 @@ namespace {
 constexpr int kFxThreads = 512;
 constexpr int kVBad = 0x7fffffff;      // digit of a potential outside the coefficient range
 constexpr int kFxStaticReserve = 4 * 1024;
+// Orbitals with a block of 4 x 4 x 4 points all 2^12 below their largest value go to the FP64 kernel: they decay
+// into a vacuum, where an FP64 stencil is right to 2^-53 of its own neighbours and a unit here is 2^-59 of the
+// largest value anywhere.  Down to 2^-12 a unit changes the exchange potential (the cube root of |u|^2) by less than
+// 2^-55 of the largest; low-pass orbitals of 9^3 to 20^3 cells and boxes have blocks of 2^-2 to 2^-9.
+constexpr int kFxRange = 12;
 
 using ll = long long;
 
@@ -322,8 +327,8 @@ __device__ __forceinline__ void fx_nonlocal_current(const FxArgs& a, const ll* p
 template <bool PER, int OBS, bool ISO, int ZL>
 __global__ void __launch_bounds__(kFxThreads, 1) k_cell_fx(FxArgs a) {
   extern __shared__ __align__(16) unsigned char fx_smem[];
-  __shared__ unsigned s_max[16], s_flag[8];
-  __shared__ unsigned s_wmax[kFxThreads / 32];
+  __shared__ unsigned s_max[8], s_min[8], s_flag[8];
+  __shared__ unsigned s_wmax[kFxThreads / 32], s_wmin[kFxThreads / 32];
   __shared__ int2 s_cd[3], s_diag;
   __shared__ int s_cbad;
   __shared__ double s_qo[3], s_jnl[3], s_obs[8][4];
@@ -353,11 +358,27 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_cell_fx(FxArgs a) {
   unsigned mx = 0;
   const int nown = (zend - zbeg) * nxy;
   double2* raw = reinterpret_cast<double2*>(buf);
-  for (int i = tid; i < nown; i += blockDim.x) {
-    const double2 u = psi[zbeg * nxy + i];
-    raw[PER ? i : (i / nxy) * ps + i % nxy] = u;
-    if (a.backup) a.backup[(size_t)orb * a.npts + zbeg * nxy + i] = u;
-    mx = max(mx, max((unsigned)__double2hiint(u.x) & 0x7fffffffu, (unsigned)__double2hiint(u.y) & 0x7fffffffu));
+  unsigned* grp = reinterpret_cast<unsigned*>(buf + slab);   // largest magnitude of four consecutive points (copy 1)
+  for (int b0 = tid; b0 < ((nown + 31) & ~31); b0 += 4 * blockDim.x) {
+    double2 u[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int i = b0 + j * (int)blockDim.x;
+      u[j] = i < nown ? psi[zbeg * nxy + i] : double2{0.0, 0.0};
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int i = b0 + j * (int)blockDim.x;
+      unsigned m = max((unsigned)__double2hiint(u[j].x) & 0x7fffffffu, (unsigned)__double2hiint(u[j].y) & 0x7fffffffu);
+      if (i < nown) {
+        raw[PER ? i : (i / nxy) * ps + i % nxy] = u[j];
+        if (a.backup) a.backup[(size_t)orb * a.npts + zbeg * nxy + i] = u[j];
+      }
+      m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+      m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
+      if ((tid & 3) == 0 && i < nown) grp[i >> 2] = m;
+      mx = max(mx, m);
+    }
   }
   mx = __reduce_max_sync(0xffffffffu, mx);
   if (lane == 0) s_wmax[warp] = mx;
@@ -393,29 +414,57 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_cell_fx(FxArgs a) {
     paddr[i] = ad;
   }
   __syncthreads();
+  // the smallest largest value of a block: four rows of four planes (of the slab; the last rows and planes where they
+  // do not divide by four) and a group of each row, the group of its x-th point
+  unsigned mn = 0x7fffffffu;
+  {
+    const int nbx = a.nx % 4 == 0 ? a.nx / 4 : (a.nx + 2) / 4 + 1, nby = (a.ny + 3) / 4, nzl = zend - zbeg;
+    for (int b = tid; b < nbx * nby * ((nzl + 3) / 4); b += blockDim.x) {
+      const int r = b / nbx, bz = r / nby, x = min(4 * (b - r * nbx), a.nx - 1);
+      const int y0 = min(4 * (r - bz * nby), a.ny - 4), z0 = max(min(4 * bz, nzl - 4), 0);
+      unsigned m = 0;
+#pragma unroll
+      for (int j = 0; j < 16; ++j) m = max(m, grp[(min(z0 + (j >> 2), nzl - 1) * nxy + (y0 + (j & 3)) * a.nx + x) >> 2]);
+      mn = min(mn, m);
+    }
+  }
+  mn = __reduce_min_sync(0xffffffffu, mn);
+  if (lane == 0) s_wmin[warp] = mn;
+  __syncthreads();
   if (ncta > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   if (warp == 0) {
-    unsigned w = lane < (int)(blockDim.x >> 5) ? s_wmax[lane] : 0u;
+    unsigned w = lane < (int)(blockDim.x >> 5) ? s_wmax[lane] : 0u, v = lane < (int)(blockDim.x >> 5) ? s_wmin[lane] : 0x7fffffffu;
     w = __reduce_max_sync(0xffffffffu, w);
+    v = __reduce_min_sync(0xffffffffu, v);
     if (lane < ncta) {
-      if (ncta > 1) st_cluster32(map_cta(smem_addr(&s_max[rank]), lane), w);
-      else s_max[0] = w;
+      if (ncta > 1) {
+        st_cluster32(map_cta(smem_addr(&s_max[rank]), lane), w);
+        st_cluster32(map_cta(smem_addr(&s_min[rank]), lane), v);
+      } else {
+        s_max[0] = w;
+        s_min[0] = v;
+      }
     }
   }
   if (ncta > 1) cluster_sync(); else __syncthreads();
   mx = 0;
-  for (int r = 0; r < ncta; ++r) mx = max(mx, s_max[r]);
+  for (int r = 0; r < ncta; ++r) {
+    mx = max(mx, s_max[r]);
+    mn = min(mn, s_min[r]);
+  }
   int e = (int)(mx >> 20);
   unsigned bad = s_cbad;
   if (mx == 0) e = 1023;
-  else if (e < 600 || e > 1450) { bad = 1; e = 1023; }
+  else if (e < 600 || e > 1450 || e - (int)(mn >> 20) > kFxRange) bad = 1;
+  if (bad) {                                       // (the same in every CTA of the cluster)
+    if (rank == 0 && tid == 0) a.need[orb] = 1;
+    return;
+  }
   const int s = 58 - (e - 1023);
   for (int i = tid; i < nown; i += blockDim.x) {
     const int li = PER ? i : (i / nxy) * ps + i % nxy;
     const double2 u = raw[li];
-    // a value far above the exponent of a flagged orbital cannot be shifted into range
-    const int2 x = bad ? make_int2(0, 0) : digits31(to_fixed(u.x, e));
-    const int2 y = bad ? make_int2(0, 0) : digits31(to_fixed(u.y, e));
+    const int2 x = digits31(to_fixed(u.x, e)), y = digits31(to_fixed(u.y, e));
     buf[li] = make_int4(x.x, x.y, y.x, y.y);
   }
   if (!PER)

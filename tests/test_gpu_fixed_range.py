@@ -1,5 +1,5 @@
 """Where the fixed-point Taylor launches of FP64 orbitals could fall short of FP64: the digits of the diagonal
-coefficient and the density of points far below an orbital's largest value."""
+coefficient, the density of points far below an orbital's largest value, and orbitals that decay into a vacuum."""
 import numpy as np
 import pytest
 
@@ -53,3 +53,31 @@ def test_diagonal_beyond_its_digits():
         ctx.taylor_step(u, 1.0, [1.4353] * 3)
         got.append(u.cpu().numpy())
     assert np.array_equal(got[0], got[1])
+
+
+def test_orbitals_in_a_vacuum():
+    """Localised orbitals in a wide box: the tail keeps FP64 accuracy (the same bits as the FP64 kernel's) and so
+    does the exchange potential, the cube root of the density (relative 1e-14: a third of the density's few units
+    and the rounding of the cube root)."""
+    s = box((20, 22, 18), (0.5,) * 3, False, 3)
+    x = [(np.arange(m) - 0.5 * (m - 1)) * 0.5 for m in s.n]
+    r2 = lambda c: (x[2][:, None, None] - c[2]) ** 2 + (x[1][:, None] - c[1]) ** 2 + (x[0] - c[0]) ** 2
+    u0 = np.stack([np.exp(-r2(c) / (2 * 0.6 ** 2)) * (1 + 0.1j) for c in ((0, 0, 0), (1, 0.5, -1), (-1, 1, 0))])[None]
+    u0 /= np.sqrt((np.abs(u0) ** 2).sum((-3, -2, -1), keepdims=True) * s.dV)
+    res = []
+    for scheme in (None, 0):
+        ctx = tdks.Context(s, precision="f64", hartree=False)
+        if scheme is not None:
+            ctx.cell_variant(scheme)
+        u = torch.from_numpy(u0).cuda()
+        ctx.update_potential(u)
+        ctx.taylor_step(u, 0.02)
+        w = torch.from_numpy(u0).cuda()
+        ctx.step(w, 0.0, 0.02)
+        res.append((u.cpu().numpy(), w.cpu().numpy(), ctx.grid_array(1).cpu().numpy()))
+    assert np.array_equal(res[0][0], res[1][0])
+    w, v = res[0][1:]
+    rho = 2 * (w.real ** 2 + w.imag ** 2).sum((0, 1))
+    assert rho.min() < 1e-25 * rho.max()
+    assert np.abs(v / (-np.cbrt(3 / np.pi * rho)) - 1).max() < 1e-14
+    assert np.abs(v - res[1][2]).max() < 1e-14 * np.abs(v).max()
