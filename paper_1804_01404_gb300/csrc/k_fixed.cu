@@ -184,9 +184,16 @@ struct DerSum {
   }
 };
 
-// Sums over points of |u|^2 (u >> 8) and Im(conj(u) D1_a u) (u >> 8 times the scaled D1 >> 6), as the
-// three sums of digit products: 2^54 v[0] + 2^27 v[1] + v[2] (the norm's middle one twice).  The shifts
-// keep the sum of a warp's points in 64 bits.
+// x >> 4 (rounded, |x| < 2^60) in digits of 28 bits: 56 bits of an orbital's largest value
+__device__ __forceinline__ int2 digits28s(ll x) {
+  const ll y = (x + 8) >> 4;
+  const int l = ((int)((unsigned)y << 4)) >> 4;
+  return make_int2((int)((y - l) >> 28), l);
+}
+// Sums over points of |u|^2 and Im(conj(u) D1_a u), of u >> 4 and the scaled D1 >> 4, as the three sums of digit
+// products: 2^56 v[0] + 2^28 v[1] + v[2] (the norm's middle one twice).  A product of digits is below 2^56 and a point
+// adds at most four, so that 32 points of a thread stay in 64 bits; parts() then carries, and the sums over
+// threads are exact.
 struct ObsAcc {
   ll n[3] = {0, 0, 0}, j[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
   __device__ __forceinline__ void norm(int2 ux, int2 uy) {
@@ -195,10 +202,20 @@ struct ObsAcc {
     n[2] = mw(ux.y, ux.y, mw(uy.y, uy.y, n[2]));
   }
   __device__ __forceinline__ void cur(int a, int2 ux, int2 uy, const ll der[2]) {
-    const int2 d0 = digits27<6>(der[0]), d1 = digits27<6>(der[1]);
+    const int2 d0 = digits28s(der[0]), d1 = digits28s(der[1]);
     j[a][0] = mw(ux.x, d0.x, mw(uy.x, d1.x, j[a][0]));
     j[a][1] = mw(ux.x, d0.y, mw(ux.y, d0.x, mw(uy.x, d1.y, mw(uy.y, d1.x, j[a][1]))));
     j[a][2] = mw(ux.y, d0.y, mw(uy.y, d1.y, j[a][2]));
+  }
+  // 2^56 v0 + 2^28 v1 + v2 = 2^84 t[0] + 2^56 t[1] + 2^28 t[2] + t[3], 0 <= t[1], t[2], t[3] < 2^28
+  static __device__ __forceinline__ void parts(ll v0, ll v1, ll v2, ll* t) {
+    const ll mask = (1 << 28) - 1;
+    t[3] = v2 & mask;
+    v1 += v2 >> 28;
+    t[2] = v1 & mask;
+    v0 += v1 >> 28;
+    t[1] = v0 & mask;
+    t[0] = v0 >> 28;
   }
 };
 
@@ -524,8 +541,8 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_cell_fx(FxArgs a) {
           const int4 u = w[zz + 4];
           int2 ux, uy;
           if (ACC) {
-            ux = digits27<8>(join31(u.x, u.y));
-            uy = digits27<8>(join31(u.z, u.w));
+            ux = digits28s(join31(u.x, u.y));
+            uy = digits28s(join31(u.z, u.w));
             oa.norm(ux, uy);
           }
           LapSum lap;
@@ -650,7 +667,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_cell_fx(FxArgs a) {
       if (d != 0.0) atomicAdd(rho + pg, __hiloint2double(__double2hiint(d) - 2 * k2 * (1 << 20), __double2loint(d)) * rfac);
     }
     if (OBS == 1) {
-      const int2 ux = digits27<8>(X), uy = digits27<8>(Y);
+      const int2 ux = digits28s(X), uy = digits28s(Y);
       oa.norm(ux, uy);
       const int y = col / a.nx, x = col - y * a.nx, z = zbeg + zz;
       const int4* p = v + zz * ps;
@@ -682,9 +699,11 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_cell_fx(FxArgs a) {
   }
   if (OBS == 0) return;
   if (OBS == 1 && a.natom > 0) fx_project<4>(a, v, pbase, pho, parto, rank, ncta, false);
-  // sums of the CTA, then of the cluster (CTA 0): integers within a warp, FP64 from there
-  ll t16[16] = {oa.n[0], oa.n[1], oa.n[2], 0, oa.j[0][0], oa.j[0][1], oa.j[0][2], 0,
-                oa.j[1][0], oa.j[1][1], oa.j[1][2], 0, oa.j[2][0], oa.j[2][1], oa.j[2][2], 0};
+  // sums of the CTA, then of the cluster (CTA 0): integers within a warp (below 2^53, so exact in FP64), FP64 from there
+  ll t16[16];
+  ObsAcc::parts(oa.n[0], 2 * oa.n[1], oa.n[2], t16);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) ObsAcc::parts(oa.j[d][0], oa.j[d][1], oa.j[d][2], t16 + 4 * (d + 1));
   const ll tw = warp_split_sum<16>(t16);           // lane L: total of value L >> 1
   if ((lane & 1) == 0) s_red[warp][lane >> 1] = tw;
   __syncthreads();
@@ -692,7 +711,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_cell_fx(FxArgs a) {
     const int q = tid & 3;
     double x = 0.0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) x += (double)s_red[w][tid];
-    x *= q == 0 ? pow2d(54) : (q == 1 ? (tid < 4 ? pow2d(28) : pow2d(27)) : 1.0);
+    x *= pow2d(28 * (3 - q));
     x += __shfl_xor_sync(0xffffu, x, 1);
     x += __shfl_xor_sync(0xffffu, x, 2);
     if (q == 0) {
@@ -712,8 +731,8 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_cell_fx(FxArgs a) {
       n += s_obs[r][0];
       if (tid >= 1 && tid < 4) x += s_obs[r][tid];
     }
-    const double sc = f1 * f1 * pow2d(14);         // u >> 8, D1 >> 6
-    n *= 4.0 * sc;
+    const double sc = f1 * f1 * pow2d(8);          // u >> 4, D1 >> 4
+    n *= sc;
     double res = 0.0;
     if (tid == 0) res = n * a.dV;
     else if (tid < 4) res = (x * sc * a.obs_fac[tid - 1] + s_qo[tid - 1] * n) * a.dV;

@@ -1,5 +1,6 @@
 """Where the fixed-point Taylor launches of FP64 orbitals could fall short of FP64: the digits of the diagonal
-coefficient, the density of points far below an orbital's largest value, and orbitals that decay into a vacuum."""
+coefficient, the density of points far below an orbital's largest value, orbitals that decay into a vacuum, and the
+current."""
 import numpy as np
 import pytest
 
@@ -81,3 +82,31 @@ def test_orbitals_in_a_vacuum():
     assert rho.min() < 1e-25 * rho.max()
     assert np.abs(v / (-np.cbrt(3 / np.pi * rho)) - 1).max() < 1e-14
     assert np.abs(v - res[1][2]).max() < 1e-14 * np.abs(v).max()
+
+
+def test_current_no_further_off_than_fp64():
+    """J of a step against sums in extended precision over the orbital it returns, the mean over 48 single orbitals:
+    no larger an error than the FP64 kernel's."""
+    ld = np.longdouble
+    d1 = [ld(4) / 5, -ld(1) / 5, ld(4) / 105, -ld(1) / 280]
+    err = {None: [], 0: []}
+    for at_start in (False, True):
+        s = box((9, 10, 11), (0.5, 0.45, 0.4), True, 1)
+        ctxs = {}
+        for scheme in err:
+            ctxs[scheme] = tdks.Context(s, precision="f64", obs_at_start=at_start)
+            if scheme is not None:
+                ctxs[scheme].cell_variant(scheme)
+        for seed in range(24):
+            u0 = W.initial_orbitals(s, seed)
+            for scheme, ctx in ctxs.items():
+                u = torch.from_numpy(u0).cuda()
+                ctx.update_potential(u)
+                ctx.step(u, 0.0, 0.02)
+                v = (u0 if at_start else u.cpu().numpy())[0, 0].astype(np.clongdouble)
+                norm = (v.real ** 2 + v.imag ** 2).sum()
+                for a in range(3):
+                    D = sum(d1[m - 1] / ld(s.h[a]) * (np.roll(v, -m, 2 - a) - np.roll(v, m, 2 - a)) for m in range(1, 5))
+                    J = -2 * (v.conj() * D).imag.sum() * ld(s.dV) / ld(s.dV * s.npts)
+                    err[scheme].append(float(abs(ctx.read_step_observables()["J"][a] - J) / (norm / s.npts)))
+    assert np.mean(err[None]) <= np.mean(err[0]), (np.mean(err[None]), np.mean(err[0]))
