@@ -93,8 +93,11 @@ struct Acc4 {
     a3 = mw(pl, ch, a3);
     a4 = mw(pl, cl, a4);
   }
-  __device__ __forceinline__ ll value(int sh) const {       // 31 < sh < 59
-    return (a1 << (59 - sh)) + (a2 >> (sh - 31)) + (a3 >> (sh - 28)) + (a4 >> sh);
+  // 31 < sh < 59.  Rounded: every lane of every CTA gives one value of a projection, and 256 floors of its three lower
+  // sums were a bias of 400 units, 3e-17 of the density in the current.
+  __device__ __forceinline__ ll value(int sh) const {
+    const ll t = a2 + ((a3 + (a4 >> 28)) >> 3);
+    return (a1 << (59 - sh)) + ((t + (1LL << (sh - 32))) >> (sh - 31));
   }
 };
 
@@ -184,7 +187,8 @@ struct DerSum {
   }
 };
 
-// x >> 4 (rounded, |x| < 2^60) in digits of 28 bits: 56 bits of an orbital's largest value
+// x >> 4 (rounded, |x| < 2^60) in digits of 28 bits: 56 bits of an orbital's largest value.  Rounding half up lifts
+// the mean by half a unit of x, which for the derivative sums meets the half unit their floor (DerSum::get) took.
 __device__ __forceinline__ int2 digits28s(ll x) {
   const ll y = (x + 8) >> 4;
   const int l = ((int)((unsigned)y << 4)) >> 4;

@@ -84,14 +84,30 @@ def test_orbitals_in_a_vacuum():
     assert np.abs(v - res[1][2]).max() < 1e-14 * np.abs(v).max()
 
 
-def test_current_no_further_off_than_fp64():
+@pytest.mark.parametrize("n,natom", [((9, 10, 11), 0), ((12, 13, 14), 3)], ids=str)
+def test_current_no_further_off_than_fp64(n, natom):
     """J of a step against sums in extended precision over the orbital it returns, the mean over 48 single orbitals:
     no larger an error than the FP64 kernel's."""
     ld = np.longdouble
     d1 = [ld(4) / 5, -ld(1) / 5, ld(4) / 105, -ld(1) / 280]
+    h = (0.5, 0.45, 0.4)
+    L = np.array(n) * h
+    atoms = [W.Atom(tuple(np.array(f) * L), 4.0) for f in ((0.21, 0.33, 0.4), (0.7, 0.64, 0.18), (0.45, 0.9, 0.77))[:natom]]
+    proj = W.Projectors()
+    tabs = []                                            # grid points, displacements and s, p projectors of an atom
+    for at in atoms:
+        d = [np.arange(n[a]) * h[a] - at.R[a] for a in range(3)]
+        d = [x - l * np.round(x / l) for x, l in zip(d, L)]
+        r2 = d[2][:, None, None] ** 2 + d[1][:, None] ** 2 + d[0] ** 2
+        iz, iy, ix = np.nonzero(r2 < proj.r_cut ** 2)
+        dd = np.stack([d[0][ix], d[1][iy], d[2][iz]])
+        r2 = r2[iz, iy, ix]
+        g = np.exp(-r2 / (2 * proj.width ** 2)) * (1 - r2 / proj.r_cut ** 2) ** 2
+        b = np.stack([g, *(dd * g)])
+        tabs.append(((iz, iy, ix), dd.astype(ld), (b / np.sqrt((b ** 2).sum(1, keepdims=True) * np.prod(h))).astype(ld)))
     err = {None: [], 0: []}
     for at_start in (False, True):
-        s = box((9, 10, 11), (0.5, 0.45, 0.4), True, 1)
+        s = box(n, h, True, 1, atoms, proj)
         ctxs = {}
         for scheme in err:
             ctxs[scheme] = tdks.Context(s, precision="f64", obs_at_start=at_start)
@@ -105,8 +121,15 @@ def test_current_no_further_off_than_fp64():
                 ctx.step(u, 0.0, 0.02)
                 v = (u0 if at_start else u.cpu().numpy())[0, 0].astype(np.clongdouble)
                 norm = (v.real ** 2 + v.imag ** 2).sum()
+                J = ctx.read_step_observables()["J"]
                 for a in range(3):
-                    D = sum(d1[m - 1] / ld(s.h[a]) * (np.roll(v, -m, 2 - a) - np.roll(v, m, 2 - a)) for m in range(1, 5))
-                    J = -2 * (v.conj() * D).imag.sum() * ld(s.dV) / ld(s.dV * s.npts)
-                    err[scheme].append(float(abs(ctx.read_step_observables()["J"][a] - J) / (norm / s.npts)))
+                    D = sum(d1[m - 1] / ld(h[a]) * (np.roll(v, -m, 2 - a) - np.roll(v, m, 2 - a)) for m in range(1, 5))
+                    ref = (v.conj() * D).imag.sum()
+                    for at, (idx, dd, b) in enumerate(tabs):
+                        f = v[idx]
+                        for p in range(4):
+                            E = proj.E_s if p == 0 else proj.E_p
+                            ref += 2 * ld(E) * ((dd[a] * b[p] * f).sum().conj() * (b[p] * f).sum()).imag * ld(s.dV)
+                    ref *= -2 * ld(s.dV) / ld(s.dV * s.npts)
+                    err[scheme].append(float(abs(J[a] - ref) / (norm / s.npts)))
     assert np.mean(err[None]) <= np.mean(err[0]), (np.mean(err[None]), np.mean(err[0]))
