@@ -32,6 +32,8 @@ namespace {
 constexpr int kMbjThreads = 128;          // k_tau, a group of k_tau_seg
 constexpr int kTauGroups = 3;             // k_tau_seg: orbital groups of a CTA (its registers fill an SM)
 constexpr int kTauSeg = 4;                // k_tau_seg: planes of a thread
+constexpr int kTauChain = 16;             // k_tau_seg: orbitals of a register sum
+constexpr size_t kTauSmem = sizeof(float) * kTauGroups * 10 * kTauSeg * kMbjThreads;
 constexpr int kBrPoints = 64;             // k_mbj_x: points of a CTA, four threads each
 constexpr double kPi23 = 2.14502939711102560008;   // pi^(2/3)
 constexpr double kPi = 3.14159265358979323846;
@@ -137,7 +139,9 @@ __global__ void __launch_bounds__(kMbjThreads) k_tau(const typename Cplx<T>::typ
 // loads instead of 50 for its two points.  One thread per pair (21 loads, any z) was bound by L2: a CTA's 256
 // points lie in one or two planes, and each orbital's eight planes around them came from L2 again for every CTA,
 // 13 times the orbital; the CTAs here cover four planes, 3 times.  The kTauGroups groups of a CTA take different
-// orbitals of the chunk and are added in shared memory, so that few chunks (FP64 folds) fill the SMs.
+// orbitals of the chunk and are added in shared memory, so that few chunks (FP64 folds) fill the SMs.  An FP32 sum in
+// registers ends after kTauChain orbitals and is added to the thread's in shared memory: one chain over a group's
+// 68 orbitals (1024 of 30^3) left the potential 1.3e-8 from FP64, sums by k-point 1.1e-8, this 0.7e-8.
 // 20^3, 1024 orbitals: 107 us before, 70 here (42 % of the issue slots; what is left is the latency of L2).
 // With an even nx a neighbour pair is wholly inside or wholly outside an isolated box.
 __device__ __forceinline__ float4 ld4_or_zero(const float2* f, int i) {
@@ -150,7 +154,7 @@ __global__ void __launch_bounds__(kMbjThreads* kTauGroups, 1) k_tau_seg(const fl
                                                                       const double* __restrict__ kw, D1h<float> d1,
                                                                       int ochunk, double* __restrict__ part) {
   constexpr int L = kTauSeg;
-  __shared__ float s_acc[kTauGroups - 1][10 * L][kMbjThreads];
+  extern __shared__ float tau_smem[];              // [kTauGroups][10 L][kMbjThreads] sums of a thread
   const int npts = nx * ny * nz, nxh = nx / 2, nxy = nx * ny, ncol = nxh * ny;
   const int grp = threadIdx.x / kMbjThreads, lt = threadIdx.x - grp * kMbjThreads;
   const int t = blockIdx.x * kMbjThreads + lt;
@@ -183,9 +187,21 @@ __global__ void __launch_bounds__(kMbjThreads* kTauGroups, 1) k_tau_seg(const fl
   }
   const int c0 = blockIdx.y * ochunk, c1 = min(c0 + ochunk, nk * norb), gl = (max(c1 - c0, 0) + kTauGroups - 1) / kTauGroups;
   const int o0 = c0 + grp * gl, o1 = in ? min(o0 + gl, c1) : o0;
+  float* mine = tau_smem + grp * 10 * L * kMbjThreads + lt;
   float acc[L][2][5];
 #pragma unroll
-  for (int i = 0; i < 10 * L; ++i) acc[i / 10][i / 5 % 2][i % 5] = 0.f;
+  for (int i = 0; i < 10 * L; ++i) {
+    acc[i / 10][i / 5 % 2][i % 5] = 0.f;
+    mine[i * kMbjThreads] = 0.f;
+  }
+  auto flush = [&]() {                             // a chain of FP32 sums ends
+#pragma unroll
+    for (int i = 0; i < 10 * L; ++i) {
+      mine[i * kMbjThreads] += acc[i / 10][i / 5 % 2][i % 5];
+      acc[i / 10][i / 5 % 2][i % 5] = 0.f;
+    }
+  };
+  int chain = 0;
   for (int o = o0; o < o1; ++o) {
     // (weighted orbital by orbital; the conversions of the weight and the wave vector are once per k)
     const int k = o / norb;
@@ -194,6 +210,10 @@ __global__ void __launch_bounds__(kMbjThreads* kTauGroups, 1) k_tau_seg(const fl
     const int oe = min(o1, (k + 1) * norb);
 #pragma unroll 1
     for (; o < oe; ++o) {
+      if (++chain > kTauChain) {
+        flush();
+        chain = 1;
+      }
       const float2* f = u + (size_t)o * npts;
       float4 w[L + 8];
 #pragma unroll
@@ -239,9 +259,7 @@ __global__ void __launch_bounds__(kMbjThreads* kTauGroups, 1) k_tau_seg(const fl
     }
     --o;
   }
-  if (grp > 0)
-#pragma unroll
-    for (int i = 0; i < 10 * L; ++i) s_acc[grp - 1][i][lt] = acc[i / 10][i / 5 % 2][i % 5];
+  flush();
   __syncthreads();
   if (grp > 0 || !in) return;
 #pragma unroll
@@ -250,9 +268,9 @@ __global__ void __launch_bounds__(kMbjThreads* kTauGroups, 1) k_tau_seg(const fl
     if (z0 + zz >= nz) break;
 #pragma unroll
     for (int c = 0; c < 5; ++c) {
-      double v = (double)acc[zz][pt][c];
+      double v = (double)mine[(i + c) * kMbjThreads];
 #pragma unroll
-      for (int g = 0; g < kTauGroups - 1; ++g) v += (double)s_acc[g][i + c][lt];
+      for (int g = 1; g < kTauGroups; ++g) v += (double)mine[(g * 10 * L + i + c) * kMbjThreads];
       part[((size_t)blockIdx.y * 5 + c) * npts + (size_t)(z0 + zz) * nxy + pxy + pt] = v;
     }
   }
@@ -457,9 +475,12 @@ cudaError_t launch_mbj(const typename Cplx<T>::type* u, int nk, int norb, const 
   for (int a = 0; a < 3; ++a)
     for (int m = 0; m < 4; ++m) d1.c[a][m] = (T)(kFD1[m] / h[a]);
   if constexpr (sizeof(T) == 4) {
-    if (seg)
-      k_tau_seg<<<grid, kMbjThreads * kTauGroups, 0, s>>>(u, nk, norb, n[0], n[1], n[2], periodic, kpts, kw, d1, ochunk,
-                                                          part);
+    if (seg) {
+      const cudaError_t es = cudaFuncSetAttribute(k_tau_seg, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTauSmem);
+      if (es != cudaSuccess) return es;
+      k_tau_seg<<<grid, kMbjThreads * kTauGroups, kTauSmem, s>>>(u, nk, norb, n[0], n[1], n[2], periodic, kpts, kw, d1, ochunk,
+                                                                 part);
+    }
   }
   if (!seg)
     k_tau<T><<<grid, kMbjThreads, 0, s>>>(u, nk, norb, n[0], n[1], n[2], periodic, kpts, kw, d1, ochunk, part);
