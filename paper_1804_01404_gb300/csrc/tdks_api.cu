@@ -520,6 +520,14 @@ bool slab_ranges(const ProjectorTables& T, int natom, int nxy, int ncta, int zl,
   return true;
 }
 
+// Whether an allocation failed that only serves a faster path, which the context then goes without.
+bool no_room(tdks_status s) {
+  if (s == TDKS_OK) return false;
+  cudaGetLastError();
+  g_err.clear();
+  return true;
+}
+
 // Tables and split of the slab launches of FP32 orbitals (k_slab.cu); the tuner decides whether they run.
 tdks_status slab_setup(tdks_ctx* c, const ProjectorTables& T) {
   if (!is_f32(c)) return TDKS_OK;
@@ -553,13 +561,11 @@ tdks_status slab_setup(tdks_ctx* c, const ProjectorTables& T) {
         link[T.pt_ent[e]] = int2{e + 1 < T.sp_off[q + 1] ? T.pt_ent[e + 1] : -1, e == T.sp_off[q] ? 1 : 0};
     int *ds = nullptr;
     int2 *dr = nullptr, *dl = nullptr;
-    TDKS_TRY(upload(c, &ds, sidx));
-    TDKS_TRY(upload(c, &dr, rng));
-    TDKS_TRY(upload(c, &dl, link));
+    if (no_room(upload(c, &ds, sidx)) || no_room(upload(c, &dr, rng)) || no_room(upload(c, &dl, link))) return TDKS_OK;
     A.sidx = ds; A.ent_rng = dr; A.link = dl;
   }
   if (!c->d_rho32) {                               // a tiled context has no density partials yet
-    TDKS_TRY(dalloc(c, &c->d_rho32, (size_t)c->npts * c->nk));
+    if (no_room(dalloc(c, &c->d_rho32, (size_t)c->npts * c->nk))) return TDKS_OK;
     TDKS_CUDA(cudaMemsetAsync(c->d_rho32, 0, sizeof(float) * (size_t)c->npts * c->nk, c->stream));
   }
   c->slab_ok = true;
@@ -630,15 +636,13 @@ tdks_status fx_setup(tdks_ctx* c, const ProjectorTables& T) {
       fac[i] = std::ldexp(T.E[i] * c->dV, c->fx_sN + 4 - c->fx_Kb);
       fac[4 * (size_t)c->natom + i] = std::ldexp(2.0 * T.E[i] * c->dV * c->dV, 2 * (c->fx_sN + 4 - c->fx_Kb) + 57 - Kd);
     }
-    TDKS_TRY(upload(c, &c->d_fx_beta, beta));
-    TDKS_TRY(upload(c, &c->d_fx_d, dd));
-    TDKS_TRY(upload(c, &c->d_fx_rng, rng));
-    TDKS_TRY(upload(c, &c->d_fx_sp, spr));
-    TDKS_TRY(upload(c, &c->d_fx_fac, fac));
-    TDKS_TRY(dalloc(c, &c->d_fx_ph, 2 * (size_t)c->ncell * c->nk * c->nsph));
+    if (no_room(upload(c, &c->d_fx_beta, beta)) || no_room(upload(c, &c->d_fx_d, dd)) ||
+        no_room(upload(c, &c->d_fx_rng, rng)) || no_room(upload(c, &c->d_fx_sp, spr)) ||
+        no_room(upload(c, &c->d_fx_fac, fac)) || no_room(dalloc(c, &c->d_fx_ph, 2 * (size_t)c->ncell * c->nk * c->nsph)))
+      return TDKS_OK;
   }
-  TDKS_TRY(dalloc(c, &c->d_fx_V, (size_t)c->npts * c->ncell));
-  TDKS_TRY(dalloc(c, &c->d_fx_need, (size_t)tot));
+  if (no_room(dalloc(c, &c->d_fx_V, (size_t)c->npts * c->ncell)) || no_room(dalloc(c, &c->d_fx_need, (size_t)tot)))
+    return TDKS_OK;
   c->fx_ok = true;
   return TDKS_OK;
 }
@@ -927,32 +931,38 @@ tdks_status tune_tile(tdks_ctx* c) {
     }
   }
   // a whole Taylor step of the tile kernels (three launches per stage, the projections beside the stencil)
-  // against one slab launch, on the zeroed orbitals
+  // against one slab launch, on zeroed orbitals: up to 304 of them (two waves of one CTA per SM), since a third set
+  // beside the work buffers may not fit; without room for those the tile kernels stay
   if (c->slab_ok && err == cudaSuccess) {
+    const int norb = c->norb;
+    c->norb = std::min(norb, std::max(1, 304 / c->nk));
+    const size_t bytes = (size_t)c->npts * c->nk * c->norb * csz;
     float ms[2] = {0.f, 0.f};
     tdks_status st = TDKS_OK;
     void* in = nullptr;
-    err = cudaMalloc(&in, n * csz);
-    if (err == cudaSuccess) err = cudaMemsetAsync(in, 0, n * csz, c->stream);
-    for (int w = 0; w < 2 && err == cudaSuccess && st == TDKS_OK; ++w) {
-      for (int r = -1; r < 3 && err == cudaSuccess && st == TDKS_OK; ++r) {
-        if (r == 0) err = cudaEventRecord(e0, c->stream);
+    cudaError_t es = cudaMalloc(&in, bytes);
+    if (es == cudaSuccess) es = cudaMemsetAsync(in, 0, bytes, c->stream);
+    for (int w = 0; w < 2 && es == cudaSuccess && st == TDKS_OK; ++w) {
+      for (int r = -1; r < 3 && es == cudaSuccess && st == TDKS_OK; ++r) {
+        if (r == 0) es = cudaEventRecord(e0, c->stream);
         if (w == 0) {
           st = tiled_kernel<float>(c, 1, in, nullptr, 0.02, nullptr, 0);
         } else {
           SlabArgs sa = c->slab;
           sa.o = make_args<float>(c, in, nullptr, c->d_v32, nullptr, 0.02, nullptr, 0);
-          if (err == cudaSuccess) err = launch_slab(sa, c->stream);
+          if (es == cudaSuccess) es = launch_slab(sa, c->stream);
         }
       }
-      if (err == cudaSuccess) err = cudaEventRecord(e1, c->stream);
-      if (err == cudaSuccess) err = cudaEventSynchronize(e1);
-      if (err == cudaSuccess) err = cudaEventElapsedTime(&ms[w], e0, e1);
+      if (es == cudaSuccess) es = cudaEventRecord(e1, c->stream);
+      if (es == cudaSuccess) es = cudaEventSynchronize(e1);
+      if (es == cudaSuccess) es = cudaEventElapsedTime(&ms[w], e0, e1);
     }
     cudaStreamSynchronize(c->stream);
     cudaFree(in);
+    c->norb = norb;
     if (st != TDKS_OK) { cudaEventDestroy(e0); cudaEventDestroy(e1); return st; }
-    c->slab_on = err == cudaSuccess && ms[1] < ms[0];
+    if (es != cudaSuccess) cudaGetLastError();
+    c->slab_on = es == cudaSuccess && ms[1] < ms[0];
     c->launches = 0;
     std::memset(c->calls, 0, sizeof(c->calls));
   }
@@ -1008,11 +1018,18 @@ tdks_status tune_cell(tdks_ctx* c) {
   c->cell_variant = 0;
   c->cell_ms[0] = c->cell_ms[1] = c->cell_ms[2] = c->cell_ms[3] = -1.f;
   if (c->tiled || (!cell_ip_ok(c) && !cell_geom_ok(c) && !c->slab_ok)) return TDKS_OK;
-  const int cell_orb = c->nk * c->norb, tnorb = std::min(c->norb, std::max(1, 1216 / c->nk));
-  const int tcell = std::max(1, std::min(c->ncell, 1216 / cell_orb)), nsub = tcell * c->nk * tnorb;
+  // at most 1216 orbitals, fewer where the device has no room for a copy of them; with room for none scheme 0 stays
   const size_t csz = is_f32(c) ? sizeof(float2) : sizeof(double2);
+  int tnk = std::min(c->nk, 1216), tnorb = std::min(c->norb, 1216 / tnk);
+  int tcell = tnk == c->nk && tnorb == c->norb ? std::min(c->ncell, 1216 / (tnk * tnorb)) : 1;
   void* buf = nullptr;
-  TDKS_CUDA(cudaMalloc(&buf, csz * (size_t)nsub * c->npts));
+  while (cudaMalloc(&buf, csz * (size_t)tcell * tnk * tnorb * c->npts) != cudaSuccess) {
+    cudaGetLastError();
+    int& x = tcell > 1 ? tcell : tnorb > 1 ? tnorb : tnk;
+    if (x == 1) return TDKS_OK;
+    x /= 2;
+  }
+  const int nsub = tcell * tnk * tnorb;
   cudaError_t err = cudaMemsetAsync(buf, 0, csz * (size_t)nsub * c->npts, c->stream);
   if (err == cudaSuccess)
     err = is_f32(c) ? cudaMemsetAsync(c->d_v32, 0, (size_t)c->npts * sizeof(float), c->stream)
@@ -1026,7 +1043,7 @@ tdks_status tune_cell(tdks_ctx* c) {
     auto run = [&]() -> cudaError_t {
       if (is_f32(c)) {
         auto a = make_args<float>(c, buf, buf, c->d_v32, nullptr, 0.02, nullptr, 0);
-        a.ncell = tcell; a.norb = tnorb; a.vstride = 0; a.Ap_cell = a.Ap_obs_cell = nullptr;
+        a.ncell = tcell; a.nk = tnk; a.norb = tnorb; a.vstride = 0; a.Ap_cell = a.Ap_obs_cell = nullptr;
         a.backup = nullptr;
         a.write_out = 1;
         a.rho32 = c->d_rho32;
@@ -1036,7 +1053,7 @@ tdks_status tune_cell(tdks_ctx* c) {
         return launch_smem_orbital<float>(a, 1, static_cast<float2*>(c->d_scratch), c->stream);
       }
       auto a = make_args<double>(c, buf, buf, c->d_v64, nullptr, 0.02, nullptr, 0);
-      a.ncell = tcell; a.norb = tnorb; a.vstride = 0; a.Ap_cell = a.Ap_obs_cell = nullptr;
+      a.ncell = tcell; a.nk = tnk; a.norb = tnorb; a.vstride = 0; a.Ap_cell = a.Ap_obs_cell = nullptr;
       a.backup = nullptr;
       a.write_out = 1;
       a.obs = c->d_orb_obs;
@@ -1058,20 +1075,21 @@ tdks_status tune_cell(tdks_ctx* c) {
   if (c->slab_ok && err == cudaSuccess) {          // the same launch in slabs over clusters
     SlabArgs sa = c->slab;
     sa.o = make_args<float>(c, buf, buf, c->d_v32, nullptr, 0.02, nullptr, 0);
-    sa.o.ncell = tcell; sa.o.norb = tnorb; sa.o.vstride = 0; sa.o.Ap_cell = sa.o.Ap_obs_cell = nullptr;
+    sa.o.ncell = tcell; sa.o.nk = tnk; sa.o.norb = tnorb; sa.o.vstride = 0; sa.o.Ap_cell = sa.o.Ap_obs_cell = nullptr;
     sa.o.backup = nullptr;
     sa.o.write_out = 1;
     sa.o.rho32 = c->d_rho32;
     sa.o.obs = c->d_orb_obs;
     sa.o.obs_at_start = c->opt.obs_at_start;
     float ms = 0.f;
-    err = launch_slab(sa, c->stream);
-    if (err == cudaSuccess) err = cudaEventRecord(e0, c->stream);
-    for (int r = 0; r < 2 && err == cudaSuccess; ++r) err = launch_slab(sa, c->stream);
-    if (err == cudaSuccess) err = cudaEventRecord(e1, c->stream);
-    if (err == cudaSuccess) err = cudaEventSynchronize(e1);
-    if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, e0, e1);
-    c->slab_on = err == cudaSuccess && 0.5f * ms < best;
+    cudaError_t es = launch_slab(sa, c->stream);
+    if (es == cudaSuccess) es = cudaEventRecord(e0, c->stream);
+    for (int r = 0; r < 2 && es == cudaSuccess; ++r) es = launch_slab(sa, c->stream);
+    if (es == cudaSuccess) es = cudaEventRecord(e1, c->stream);
+    if (es == cudaSuccess) es = cudaEventSynchronize(e1);
+    if (es == cudaSuccess) es = cudaEventElapsedTime(&ms, e0, e1);
+    if (es != cudaSuccess) cudaGetLastError();
+    c->slab_on = es == cudaSuccess && 0.5f * ms < best;
   }
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
