@@ -2706,6 +2706,30 @@ tdks_status tdks_set_predictor(tdks_ctx* c, int mode, double threshold) {
 }
 
 
+// The training workspace: as many samples as a batch of `want` has, the group limit and kTrainBytes allow (at
+// least one); kept in the context and grown when a larger batch comes, as far as the device has room.  tdks_nn_init
+// takes that of one sample.
+static tdks_status train_workspace(tdks_ctx* c, int want) {
+  int S = std::min(want, kTrainGroup);
+  while (S > 1 && nn_train_bytes(c->npts, S) > kTrainBytes) --S;
+  void* p = nullptr;
+  while (!c->nn.train || S > c->nn.train_S) {
+    if (cudaMalloc(&p, nn_train_bytes(c->npts, S)) == cudaSuccess) {
+      if (c->nn.train) {
+        TDKS_CUDA(cudaStreamSynchronize(c->stream));
+        cudaFree(c->nn.train);
+      }
+      c->nn.train = p;
+      c->nn.train_S = S;
+      return TDKS_OK;
+    }
+    cudaGetLastError();
+    if (S == 1) return fail(TDKS_ENOMEM, "training workspace");
+    S /= 2;
+  }
+  return TDKS_OK;
+}
+
 tdks_status tdks_nn_init(tdks_ctx* c, unsigned long long seed) {
   TDKS_TRY(check_ctx(c));
   NNBuffers& B = c->nn;
@@ -2729,6 +2753,7 @@ tdks_status tdks_nn_init(tdks_ctx* c, unsigned long long seed) {
     TDKS_TRY(dalloc(c, &wt, nn_wtrain_bytes()));
     B.wtrain = wt;
     B.err = c->d_err;
+    TDKS_TRY(train_workspace(c, 1));
   }
   std::vector<float> p(kNNParams, 0.0f);
   const int fan[3] = {4 * 27, 16 * 27, 16 * 27};
@@ -2760,32 +2785,6 @@ tdks_status tdks_nn_params(tdks_ctx* c, float* host, int n, int set) {
     TDKS_CUDA(cudaMemcpyAsync(host, c->nn.params, n * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
   }
   TDKS_CUDA(cudaStreamSynchronize(c->stream));
-  return TDKS_OK;
-}
-
-// The training workspace: as many samples as a batch of `want` has, the group limit and kTrainBytes allow (at
-// least one); kept in the context and grown when a larger batch comes.
-static tdks_status train_workspace(tdks_ctx* c, int want) {
-  int S = std::min(want, kTrainGroup);
-  while (S > 1 && nn_train_bytes(c->npts, S) > kTrainBytes) --S;
-  if (c->nn.train && c->nn.train_S >= S) return TDKS_OK;
-  if (c->nn.train) {
-    TDKS_CUDA(cudaStreamSynchronize(c->stream));
-    cudaFree(c->nn.train);
-    c->nn.train = nullptr;
-  }
-  cudaError_t e = cudaMalloc(&c->nn.train, nn_train_bytes(c->npts, S));
-  while (e != cudaSuccess && S > 1) {
-    cudaGetLastError();
-    S /= 2;
-    e = cudaMalloc(&c->nn.train, nn_train_bytes(c->npts, S));
-  }
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    c->nn.train = nullptr;
-    return fail(TDKS_ENOMEM, "training workspace");
-  }
-  c->nn.train_S = S;
   return TDKS_OK;
 }
 

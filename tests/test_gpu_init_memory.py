@@ -41,3 +41,36 @@ def test_set_up_with_little_room(n, periodic, norb):
     finally:
         del fill
         torch.cuda.empty_cache()
+
+
+def test_training_after_the_device_filled_up():
+    """The predictor's set-up takes what training one sample at a time needs; a device that is full afterwards only
+    costs the larger groups."""
+    s = W.tiny(periodic=True, n=(12, 12, 12), norb=2, natom=1)
+    ctx = tdks.Context(s, precision="f32")
+    g = torch.Generator("cuda").manual_seed(1)
+    v = torch.randn((40, 12, 12, 12), generator=g, dtype=torch.float64, device="cuda")
+    ctx.nn_init(0)
+    p = ctx.nn_params()
+    want = ctx.nn_train(v, epochs=1, batch=8, lr=1e-3, seed=0), ctx.nn_params()
+    ctx.close()
+    ctx = tdks.Context(s, precision="f32")
+    ctx.nn_init(0)
+    ctx.nn_params(p)
+    fill = []
+    for size in (1 << 34, 1 << 30, 1 << 26, 1 << 22, 2 * MiB):
+        while True:
+            try:
+                fill.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+            except torch.OutOfMemoryError:
+                break
+    try:
+        loss, grad = ctx.nn_gradient(v[1:5], v[5])
+        got = ctx.nn_train(v, epochs=1, batch=8, lr=1e-3, seed=0), ctx.nn_params()
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    assert np.isfinite(loss) and np.isfinite(grad).all()
+    # the same samples in groups of other sizes: FP32 sums in another order, then Adam's normalised step of 1e-3
+    assert np.allclose(got[0], want[0], rtol=1e-5)
+    assert np.linalg.norm(got[1] - want[1]) < 1e-4 * np.linalg.norm(want[1])
