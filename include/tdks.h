@@ -429,9 +429,11 @@ tdks_status tdks_query(const tdks_ctx* ctx, int* npts, int* nk, int* norb, int* 
  * 2 CTAs per SM, prefetch 8; 4 = the same with 4 consumer warps and 4 CTAs per SM; 5, 6 = 3, 4 with
  * the potential (and for a Horner stage psi) of each plane delivered by TMA next to the orbital
  * plane instead of loaded per thread (grids with nx divisible by 4).  FP64: 0 and 1 (one CTA per SM,
- * without / with prefetch).
- *   set       : -1 leaves the choice as it is; 0..6 forces that variant for both uses.
- *   variant   : receives the variants in use [H v, Horner stage] (may be NULL).
+ * without / with prefetch).  H v always uses these kernels; Taylor launches of FP32 orbitals may run as
+ * slab launches instead (tdks_taylor_path).
+ *   set       : -1 leaves the choice as it is; 0..6 forces that variant for both uses and the tile
+ *               kernels for the Taylor launches (TDKS_PATH_KERNELS).
+ *   variant   : receives the variants [H v, Horner stage] of the tile kernels (may be NULL).
  *   tune_ms   : receives the 14 tuning times in ms [use][variant], -1 where not timed (may be NULL).
  * Errors: EUNSUPPORTED if the context does not use the tile kernels or the variant does not apply
  * (FP32 only; nx % 4 for 5 and 6); EINVAL for set outside -1..6. */
@@ -460,13 +462,35 @@ tdks_status tdks_project_variant(tdks_ctx* ctx, int set, int* variant, float* tu
  * (FP32 only).  The arithmetic per grid point and per projection is the same in all four; the norm and
  * current sums of an orbital are split over the CTA's warps and may add in another order.  At
  * tdks_init a cell context on which scheme 1, 2 or 3 applies times one Taylor launch of each scheme
- * that applies on zeroed orbitals and keeps the fastest.
- *   set       : -1 leaves the choice as it is; 0..3 forces that scheme.
- *   variant   : receives the scheme in use (may be NULL).
+ * that applies on zeroed orbitals and keeps the fastest.  The Taylor launches run in that scheme where
+ * tdks_taylor_path says TDKS_PATH_KERNELS; FP64 orbitals that leave the range of the fixed-point
+ * launches also run in it.
+ *   set       : -1 leaves the choice as it is; 0..3 forces that scheme, and TDKS_PATH_KERNELS
+ *               (tdks_taylor_path with TDKS_PATH_AUTO goes back).
+ *   variant   : receives the scheme (may be NULL).
  *   tune_ms   : receives the 4 tuning times in ms, -1 where not timed (may be NULL).
  * Errors: EUNSUPPORTED if the context uses the tile kernels, or set = 1, 2 or 3 where that scheme
  * does not apply; EINVAL for set outside -1..3. */
 tdks_status tdks_cell_variant(tdks_ctx* ctx, int set, int* variant, float* tune_ms);
+
+/* Kernels of the Taylor launches (tdks_step, tdks_taylor_step, tdks_ms_step; no counterpart in the paper).
+ * TDKS_PATH_KERNELS: the cell kernels in the scheme of tdks_cell_variant, or the tile kernels.
+ * TDKS_PATH_SLAB: an FP32 orbital in slabs over the shared memory of one to eight SMs; the same sums per
+ * grid point, the projections' added in another order.
+ * TDKS_PATH_FIXED: an FP64 orbital of a cell context as 64-bit integers with one scale, 2^-59 of its largest
+ * value a unit, over one to eight SMs.  Orbitals that do not fit that -- not finite, beyond 2^+-423,
+ * 2^12 below their largest value in whole blocks of 4 x 4 x 4 points, a time step or a wave vector
+ * beyond the coefficients -- are propagated by the cell kernels, in the same call.
+ * At tdks_init FP64 cell contexts that can take TDKS_PATH_FIXED do; FP32 contexts that can take
+ * TDKS_PATH_SLAB time one launch of it (tiled contexts: four Taylor steps of up to 304 orbitals) against
+ * the other kernels and keep the faster.  That and the schemes' trial runs are most of tdks_init: 3 to 8 ms
+ * in FP32, 54 ms for 1024 FP64 orbitals of 20^3.
+ *   set   : -1 leaves the path as it is; TDKS_PATH_AUTO goes back to the choice of tdks_init (the
+ *           scheme of tdks_cell_variant stays as it was set); the others force that path.
+ *   path  : receives the path in use, 1..3 (may be NULL).
+ * Errors: EUNSUPPORTED for a path the context cannot take; EINVAL for set outside -1..3. */
+enum { TDKS_PATH_AUTO = 0, TDKS_PATH_KERNELS = 1, TDKS_PATH_SLAB = 2, TDKS_PATH_FIXED = 3 };
+tdks_status tdks_taylor_path(tdks_ctx* ctx, int set, int* path);
 
 /* Checkpoint and restart of the time stepping (no counterpart in the paper's formulation; the
  * paper's code restarts from files).  The state is everything a context carries from step to step
@@ -511,7 +535,8 @@ tdks_status tdks_set_wait_test(tdks_ctx* ctx, long long wait_limit, int stop_aft
  * control, loops that must never allocate -- this
  * computes vhxc = V_H[rho] + V_xc[rho] (hartree / xc select the terms, as in tdks_options; xc = 3,
  * TB-mBJ, needs the orbitals and returns TDKS_EINVAL here) for a
- * periodic or isolated grid with the same kernels as tdks_update_potential, using a fixed work area
+ * periodic or isolated grid like tdks_update_potential (which transforms isolated grids and batches of cells in
+ * 64-bit fixed point up to 256 points, where this runs FP64 lines; they agree to rounding), using a fixed work area
  * built into the library (6 MiB of device memory per GPU that loads the library, held until the
  * process exits) instead of context buffers.  rho_dev and vhxc_dev are caller-owned device arrays
  * [nz][ny][nx] of doubles; stream is a cudaStream_t (NULL = legacy default stream); the call is

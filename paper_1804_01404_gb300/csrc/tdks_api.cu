@@ -97,14 +97,14 @@ struct tdks_ctx {
   double *d_beta64 = nullptr, *d_d64 = nullptr, *d_E64 = nullptr;
   float *d_beta32 = nullptr, *d_d32 = nullptr, *d_E32 = nullptr;
   double *d_kpts = nullptr, *d_kw = nullptr;
+  int path = TDKS_PATH_AUTO;     // tdks_taylor_path; a cell or tile variant that is set makes it TDKS_PATH_KERNELS
   // Taylor launches of FP32 orbitals in slabs over a cluster (k_slab.cu): the split, whether the grid allows
-  // them, whether the tuner kept them, and whether a cell or tile variant that was set turned them off
+  // them, whether the tuner kept them
   SlabArgs slab{};
-  bool slab_ok = false, slab_on = false, slab_forced_off = false;
+  bool slab_ok = false, slab_on = false;
   // fixed-point Taylor launches of FP64 orbitals (k_fixed.cu): split of an orbital over a cluster, digit
   // tables of the projectors, digits of the step potential and of the phases, per-orbital range flags
   bool fx_ok = false;            // the grid, the projectors and the options allow it
-  bool fx_forced_off = false;    // tdks_cell_variant has set an FP64 scheme
   int fx_ncta = 1, fx_zl = 0, fx_zlen = 0, fx_nseg = 0, fx_sN = 0, fx_Kb = 0;
   double fx_nl_bound = 0.0;      // largest row sum of |V_NL| and of |E_p dV beta|
   int4 *d_fx_beta = nullptr, *d_fx_ph = nullptr;
@@ -391,7 +391,7 @@ struct Phase {
 // V used by the next orbital kernel: V_loc + a * V_Hxc + b * V_pred
 // Whether the density of an orbital kernel is written whole (FP32 cell kernels: per-k partials folded
 // into rho) rather than accumulated into a zeroed rho (FP64 atomics, the tile path).
-bool slab_use(const tdks_ctx* c) { return c->slab_on && !c->slab_forced_off; }
+bool slab_use(const tdks_ctx* c) { return c->path == TDKS_PATH_AUTO ? c->slab_on : c->path == TDKS_PATH_SLAB; }
 bool rho_overwritten(const tdks_ctx* c) { return is_f32(c) && (!c->tiled || slab_use(c)); }
 
 tdks_status set_step_potential(tdks_ctx* c, double a, const double* v2, double b) {
@@ -689,10 +689,16 @@ FxArgs make_fx_args(const tdks_ctx* c, const OrbArgs<double>& o) {
 // Whether a Taylor launch of step dt runs in fixed point: the weights of the step stay in the range of
 // its coefficients (the kernel checks the wave vector, the potential and the orbital themselves).
 bool fx_use(const tdks_ctx* c, double dt) {
-  if (!c->fx_ok || c->fx_forced_off || !std::isfinite(dt)) return false;
+  if (!c->fx_ok || c->path == TDKS_PATH_KERNELS || !std::isfinite(dt)) return false;
   double s = 0.0;
   for (int d = 0; d < 3; ++d) s += (3.251 + 1.4237) / (c->grid.h[d] * c->grid.h[d]);
   return std::fabs(dt) * s < 4.0 && std::fabs(dt) * c->fx_nl_bound < 0.9;
+}
+
+// the path of the Taylor launches (of a usual step)
+int taylor_path(const tdks_ctx* c) {
+  if (slab_use(c)) return TDKS_PATH_SLAB;
+  return c->fx_ok && c->path != TDKS_PATH_KERNELS ? TDKS_PATH_FIXED : TDKS_PATH_KERNELS;
 }
 
 // phase: profiling phase (-1: H u -> hpsi, a written Taylor result -> corrector, else predictor)
@@ -2317,7 +2323,7 @@ static tdks_status predicted_step(tdks_ctx* c, void* u, const double Amid[3], co
   tdks_ctx::StepKey key;
   key.u = u; key.dt = dt; key.thr = c->pred_thr; key.mbj_c = c->mbj_c_fixed; key.mode = c->pred_mode;
   key.lg = c->longitudinal ? 1 : 0; key.has_obs = Aobs ? 1 : 0; key.obs_start = obs_start ? 1 : 0;
-  key.cell_variant = c->cell_variant + (c->fx_forced_off ? 16 : 0) + (slab_use(c) ? 32 : 0); key.tile0 = c->tile_variant[0]; key.tile1 = c->tile_variant[1];
+  key.cell_variant = c->cell_variant + 16 * taylor_path(c); key.tile0 = c->tile_variant[0]; key.tile1 = c->tile_variant[1];
   key.prof = c->profiling ? (c->prof_stencil_only ? 2 : 1) : 0;
   key.proj = c->proj_variant;
   if (!(key == c->sg_key)) {
@@ -2502,7 +2508,7 @@ tdks_status tdks_ms_step(tdks_ctx* c, void* u, double t, double dt) {
   if (c->step_graph && c->ms_steps > 0) {
     // a replay of the step's graph: one launch, no host work between the kernels
     tdks_ctx::MsKey key;
-    key.u = u; key.dt = dt; key.mbj_c = c->mbj_c_fixed; key.cell_variant = c->cell_variant + (c->fx_forced_off ? 16 : 0) + (slab_use(c) ? 32 : 0);
+    key.u = u; key.dt = dt; key.mbj_c = c->mbj_c_fixed; key.cell_variant = c->cell_variant + 16 * taylor_path(c);
     key.tile0 = c->tile_variant[0]; key.tile1 = c->tile_variant[1];
     key.prof = c->profiling ? (c->prof_stencil_only ? 2 : 1) : 0;
     if (!(key == c->msg_key)) {
@@ -2923,7 +2929,7 @@ tdks_status tdks_tile_variant(tdks_ctx* c, int set, int* variant, float* tune_ms
     return fail(TDKS_EUNSUPPORTED, "tile variants 5 and 6 need nx divisible by 4");
   if (set >= 0) {
     c->tile_variant[0] = c->tile_variant[1] = set;
-    c->slab_forced_off = true;                      // the tile kernels run
+    c->path = TDKS_PATH_KERNELS;
   }
   if (variant) { variant[0] = c->tile_variant[0]; variant[1] = c->tile_variant[1]; }
   if (tune_ms)
@@ -2946,11 +2952,23 @@ tdks_status tdks_cell_variant(tdks_ctx* c, int set, int* variant, float* tune_ms
                                    "with FP32 orbitals");
   if (set >= 0) {
     c->cell_variant = set;
-    c->fx_forced_off = c->slab_forced_off = true;   // the scheme that was set runs
+    c->path = TDKS_PATH_KERNELS;                    // the scheme that was set runs
   }
   if (variant) *variant = c->cell_variant;
   if (tune_ms)
     for (int v = 0; v < 4; ++v) tune_ms[v] = c->cell_ms[v];
+  return TDKS_OK;
+}
+
+tdks_status tdks_taylor_path(tdks_ctx* c, int set, int* path) {
+  TDKS_TRY(check_ctx(c));
+  if (set < -1 || set > TDKS_PATH_FIXED) return fail(TDKS_EINVAL, "Taylor path outside -1..3");
+  if (set == TDKS_PATH_SLAB && !c->slab_ok)
+    return fail(TDKS_EUNSUPPORTED, "slab launches need FP32 orbitals that fit the shared memory of eight SMs");
+  if (set == TDKS_PATH_FIXED && !c->fx_ok)
+    return fail(TDKS_EUNSUPPORTED, "fixed-point launches need FP64 orbitals of a cell context, in slabs of at most eight SMs");
+  if (set >= 0) c->path = set;
+  if (path) *path = taylor_path(c);
   return TDKS_OK;
 }
 

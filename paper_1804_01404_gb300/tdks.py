@@ -16,6 +16,7 @@ LIB_PATH = os.path.join(HERE, "libtdks.so")
 
 TDKS_F64, TDKS_F32 = 0, 1
 PRED_PC, PRED_EXTRAP, PRED_LEARNED = 0, 1, 2
+PATH_AUTO, PATH_KERNELS, PATH_SLAB, PATH_FIXED = 0, 1, 2, 3   # tdks_taylor_path
 STEP_OBS_DOUBLES = 11        # doubles of one step-observable block (tdks_copy_step_observables)
 NN_NPARAMS = 9105
 FIELD_NONE, FIELD_STEP, FIELD_PULSE, FIELD_TABLE = 0, 1, 2, 3
@@ -121,6 +122,7 @@ def load_library(path: str = LIB_PATH):
         "tdks_query": [vp, C.POINTER(i), C.POINTER(i), C.POINTER(i), C.POINTER(i), C.POINTER(i)],
         "tdks_tile_variant": [vp, i, C.POINTER(i), C.POINTER(C.c_float)],
         "tdks_cell_variant": [vp, i, C.POINTER(i), C.POINTER(C.c_float)],
+        "tdks_taylor_path": [vp, i, C.POINTER(i)],
         "tdks_project_variant": [vp, i, C.POINTER(i), C.POINTER(C.c_float)],
         "tdks_set_wait_test": [vp, C.c_longlong, i],
         "tdks_state_size": [vp, C.POINTER(C.c_size_t)],
@@ -542,13 +544,20 @@ class Context:
         return v.value, [float(x) for x in ms]
 
     def cell_variant(self, set=-1):
-        """Buffer scheme of the cell kernels' Taylor launches (tdks_cell_variant): returns (scheme in
-        use, tuning ms [two buffers, in-place sweep, two buffers with the grid size built in, in-place
-        sweep with the grid size built in])."""
+        """Buffer scheme of the cell kernels' Taylor launches (tdks_cell_variant): returns (scheme, tuning
+        ms [two buffers, in-place sweep, two buffers with the grid size built in, in-place sweep with the
+        grid size built in])."""
         v = C.c_int()
         ms = (C.c_float * 4)()
         _check(self.lib.tdks_cell_variant(self.ctx, int(set), C.byref(v), ms))
         return v.value, [float(x) for x in ms]
+
+    def taylor_path(self, set=-1):
+        """Kernels of the Taylor launches (tdks_taylor_path): PATH_KERNELS, PATH_SLAB or PATH_FIXED; set also
+        takes PATH_AUTO, the choice made at set-up."""
+        v = C.c_int()
+        _check(self.lib.tdks_taylor_path(self.ctx, int(set), C.byref(v)))
+        return v.value
 
     def get_state(self):
         """Checkpoint of the time-stepping state (tdks_get_state) as a numpy uint8 array."""
