@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(kSlabThreads, 2) k_slab(SlabArgs A) {
         } while (e >= 0);
         const float2 r = M::fma(coef, make_float2(im, -re), nxt[li]);
         nxt[li] = r;
-        if (PER && !EVEN && (li % ps) % nxp == 0) nxt[li + nx] = r;   // the row's pad
+        if (PER && !EVEN && nxp > nx && (li % ps) % nxp == 0) nxt[li + nx] = r;   // the row's pad (odd nx)
       }
       if (ncta > 1) cluster_sync(); else __syncthreads();
     }

@@ -15,7 +15,7 @@ MORE = [((16, 16, 16), (0.5,) * 3, True, 9, 2, 2), ((20, 20, 20), (0.5,) * 3, Tr
 
 
 @pytest.mark.parametrize("spec", SYSTEMS + MORE, ids=lambda s: "x".join(map(str, s[0])) + ("p" if s[2] else "i"))
-@pytest.mark.parametrize("at_start,off", [(False, 0), (True, 0)])
+@pytest.mark.parametrize("at_start,off", [(False, 0), (True, 0), (False, 1), (True, 1)])
 def test_forced_slabs(spec, at_start, off):
     s = system(*spec)
     u0 = orbitals(s)
