@@ -50,9 +50,7 @@ template <typename T>
 __host__ __device__ inline size_t cell_smem_bytes(int nz, int pstride, int nsph, int natom, bool dbuf) {
   using C = typename Cplx<T>::type;
   const size_t vsz = (size_t)nz * pstride;
-  // the z window prefetches plane z + 5, which after the last plane of a 4-plane cell wraps to plane 4: a
-  // plane of slack behind the copies (the value is not used; a guard in the loop cost 7 % of a launch)
-  return sizeof(C) * (vsz * (dbuf ? 2 : 1) + nsph + 4 * (size_t)natom + (nz == 4 ? pstride : 0));
+  return sizeof(C) * (vsz * (dbuf ? 2 : 1) + nsph + 4 * (size_t)natom);
 }
 
 // Threads per CTA (upper bound): 25 warps for FP32 (two z-segments per column of a 20^2 plane; the
@@ -1191,7 +1189,9 @@ __global__ void __launch_bounds__(kMaxThreads<T, IP, GEOM>(), kMinBlocks<T, IP, 
             if (DBUF) L.nxt[zb + c.col] = r; else gnxt[pg] = r;
 #pragma unroll
             for (int j = 0; j < 8; ++j) w[j] = w[j + 1];
-            w[8] = zload<T, PER>(a, L.v, z + 5, c.col);
+            // (the last plane needs none; z + 5 would wrap to a plane 4 that a 4-plane cell does not have, and a
+            // branch here cost 7 % of a launch)
+            w[8] = zload<T, PER>(a, L.v, min(z + 5, c.z1 + 3), c.col);
           }
         }
       }
@@ -1291,7 +1291,7 @@ __global__ void __launch_bounds__(kMaxThreads<T, IP, GEOM>(), kMinBlocks<T, IP, 
         }
 #pragma unroll
         for (int j = 0; j < 4; ++j) w[j] = w[j + 1];
-        w[4] = zload<T, PER>(a, L.v, z + 5, c.col);
+        w[4] = zload<T, PER>(a, L.v, min(z + 5, c.z1 + 3), c.col);
       }
     }
   }
