@@ -482,9 +482,10 @@ tdks_status tdks_cell_variant(tdks_ctx* ctx, int set, int* variant, float* tune_
  * 2^12 below their largest value in whole blocks of 4 x 4 x 4 points, a time step or a wave vector
  * beyond the coefficients -- are propagated by the cell kernels, in the same call.
  * At tdks_init FP64 cell contexts that can take TDKS_PATH_FIXED do; FP32 contexts that can take
- * TDKS_PATH_SLAB time one launch of it (tiled contexts: four Taylor steps of up to 304 orbitals) against
- * the other kernels and keep the faster.  That and the schemes' trial runs are most of tdks_init: 3 to 8 ms
- * in FP32, 54 ms for 1024 FP64 orbitals of 20^3.
+ * TDKS_PATH_SLAB time one launch of it (tiled contexts: a Taylor step of up to 304 orbitals) against the
+ * other kernels and keep the faster; cells of a built-in size (schemes 2 and 3) with 304 orbitals or more
+ * keep those.  The trial runs are most of tdks_init: 3 to 7 ms in FP32, 54 ms for 1024 FP64 orbitals of
+ * 20^3.
  *   set   : -1 leaves the path as it is; TDKS_PATH_AUTO goes back to the choice of tdks_init (the
  *           scheme of tdks_cell_variant stays as it was set); the others force that path.
  *   path  : receives the path in use, 1..3 (may be NULL).

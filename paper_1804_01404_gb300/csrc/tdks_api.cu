@@ -535,21 +535,20 @@ tdks_status slab_setup(tdks_ctx* c, const ProjectorTables& T) {
   const int nxy = n[0] * n[1];
   SlabArgs& A = c->slab;
   std::vector<int2> rng, spr;
+  std::vector<int> ent(n[2] + 1, 0);               // sphere entries below plane z
+  for (int i : T.idx) ent[i / nxy + 1] += 1;
+  for (int z = 0; z < n[2]; ++z) ent[z + 1] += ent[z];
   int max_ent[9] = {0};
-  for (int k = 1; k <= 8 && c->natom > 0; ++k) {
-    if (!slab_ranges(T, c->natom, nxy, k, (n[2] + k - 1) / k, rng, spr)) return TDKS_OK;
-    for (int r = 0; r < k; ++r) {
-      int e = 0;
-      for (int a = 0; a < c->natom; ++a) e += rng[(size_t)r * c->natom + a].y - rng[(size_t)r * c->natom + a].x;
-      max_ent[k] = std::max(max_ent[k], e);
-    }
+  for (int k = 1; k <= 8; ++k) {
+    const int zl = (n[2] + k - 1) / k;
+    for (int z = 0; z < n[2]; z += zl) max_ent[k] = std::max(max_ent[k], ent[std::min(n[2], z + zl)] - ent[z]);
     max_ent[k] = (max_ent[k] + 3) & ~3;
   }
   if (!slab_split(n[0], n[1], n[2], c->grid.periodic != 0, c->natom, max_ent, c->ncell * c->nk * c->norb, &A)) return TDKS_OK;
   if (c->natom > 0) {
     // (the kernel's tables number a CTA's entries and the atoms with 16 bits)
     if (A.max_ent > 65000 || c->natom > 65000) return TDKS_OK;
-    slab_ranges(T, c->natom, nxy, A.ncta, A.zl, rng, spr);
+    if (!slab_ranges(T, c->natom, nxy, A.ncta, A.zl, rng, spr)) return TDKS_OK;
     std::vector<int> sidx(T.idx.size());
     for (size_t i = 0; i < T.idx.size(); ++i) {
       const int z = T.idx[i] / nxy, r = T.idx[i] - z * nxy, y = r / n[0];
@@ -949,8 +948,8 @@ tdks_status tune_tile(tdks_ctx* c) {
     cudaError_t es = cudaMalloc(&in, bytes);
     if (es == cudaSuccess) es = cudaMemsetAsync(in, 0, bytes, c->stream);
     for (int w = 0; w < 2 && es == cudaSuccess && st == TDKS_OK; ++w) {
-      for (int r = -1; r < 3 && es == cudaSuccess && st == TDKS_OK; ++r) {
-        if (r == 0) es = cudaEventRecord(e0, c->stream);
+      for (int r = 0; r < 2 && es == cudaSuccess && st == TDKS_OK; ++r) {
+        if (r == 1) es = cudaEventRecord(e0, c->stream);
         if (w == 0) {
           st = tiled_kernel<float>(c, 1, in, nullptr, 0.02, nullptr, 0);
         } else {
@@ -1023,7 +1022,12 @@ bool cell_variant_ok(const tdks_ctx* c, int v) {
 tdks_status tune_cell(tdks_ctx* c) {
   c->cell_variant = 0;
   c->cell_ms[0] = c->cell_ms[1] = c->cell_ms[2] = c->cell_ms[3] = -1.f;
-  if (c->tiled || (!cell_ip_ok(c) && !cell_geom_ok(c) && !c->slab_ok)) return TDKS_OK;
+  const bool schemes = cell_ip_ok(c) || cell_geom_ok(c);
+  // the slab launch, against scheme 0 alone once each after one untimed launch; with the grid size built in only where
+  // few orbitals leave SMs idle (1024 of 20^3: 430 us in slabs, 217 with the size built in)
+  const bool slab = c->slab_ok && !(cell_geom_ok(c) && is_f32(c) && c->ncell * c->nk * c->norb >= 304);
+  if (c->tiled || (!schemes && !slab)) return TDKS_OK;
+  const int reps = schemes ? 2 : 1;
   // at most 1216 orbitals, fewer where the device has no room for a copy of them; with room for none scheme 0 stays
   const size_t csz = is_f32(c) ? sizeof(float2) : sizeof(double2);
   int tnk = std::min(c->nk, 1216), tnorb = std::min(c->norb, 1216 / tnk);
@@ -1069,16 +1073,17 @@ tdks_status tune_cell(tdks_ctx* c) {
     };
     err = run();
     if (err == cudaSuccess) err = cudaEventRecord(e0, c->stream);
-    for (int r = 0; r < 2 && err == cudaSuccess; ++r) err = run();
+    for (int r = 0; r < reps && err == cudaSuccess; ++r) err = run();
     if (err == cudaSuccess) err = cudaEventRecord(e1, c->stream);
     if (err == cudaSuccess) err = cudaEventSynchronize(e1);
     float ms = 0.f;
     if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, e0, e1);
     if (err != cudaSuccess) break;
-    if (cell_ip_ok(c) || cell_geom_ok(c)) c->cell_ms[v] = 0.5f * ms;   // (with a choice of schemes)
-    if (v == 0 || 0.5f * ms < (v == 3 && c->cell_variant == 2 ? 0.97f : 1.f) * best) { best = 0.5f * ms; c->cell_variant = v; }
+    ms /= reps;
+    if (schemes) c->cell_ms[v] = ms;               // (with a choice of schemes)
+    if (v == 0 || ms < (v == 3 && c->cell_variant == 2 ? 0.97f : 1.f) * best) { best = ms; c->cell_variant = v; }
   }
-  if (c->slab_ok && err == cudaSuccess) {          // the same launch in slabs over clusters
+  if (slab && err == cudaSuccess) {                // the same launch in slabs over clusters
     SlabArgs sa = c->slab;
     sa.o = make_args<float>(c, buf, buf, c->d_v32, nullptr, 0.02, nullptr, 0);
     sa.o.ncell = tcell; sa.o.nk = tnk; sa.o.norb = tnorb; sa.o.vstride = 0; sa.o.Ap_cell = sa.o.Ap_obs_cell = nullptr;
@@ -1090,12 +1095,12 @@ tdks_status tune_cell(tdks_ctx* c) {
     float ms = 0.f;
     cudaError_t es = launch_slab(sa, c->stream);
     if (es == cudaSuccess) es = cudaEventRecord(e0, c->stream);
-    for (int r = 0; r < 2 && es == cudaSuccess; ++r) es = launch_slab(sa, c->stream);
+    for (int r = 0; r < reps && es == cudaSuccess; ++r) es = launch_slab(sa, c->stream);
     if (es == cudaSuccess) es = cudaEventRecord(e1, c->stream);
     if (es == cudaSuccess) es = cudaEventSynchronize(e1);
     if (es == cudaSuccess) es = cudaEventElapsedTime(&ms, e0, e1);
     if (es != cudaSuccess) cudaGetLastError();
-    c->slab_on = es == cudaSuccess && 0.5f * ms < best;
+    c->slab_on = es == cudaSuccess && ms < reps * best;
   }
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
