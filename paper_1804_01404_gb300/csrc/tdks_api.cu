@@ -2719,24 +2719,26 @@ tdks_status tdks_set_predictor(tdks_ctx* c, int mode, double threshold) {
 
 // The training workspace: as many samples as a batch of `want` has, the group limit and kTrainBytes allow (at
 // least one); kept in the context and grown when a larger batch comes, as far as the device has room.  tdks_nn_init
-// takes that of one sample.
+// takes that of one sample, which is kept beside a larger one (freeing it took 60 us of the first training call).
 static tdks_status train_workspace(tdks_ctx* c, int want) {
   int S = std::min(want, kTrainGroup);
   while (S > 1 && nn_train_bytes(c->npts, S) > kTrainBytes) --S;
-  void* p = nullptr;
-  while (!c->nn.train || S > c->nn.train_S) {
-    if (cudaMalloc(&p, nn_train_bytes(c->npts, S)) == cudaSuccess) {
-      if (c->nn.train) {
-        TDKS_CUDA(cudaStreamSynchronize(c->stream));
-        cudaFree(c->nn.train);
-      }
-      c->nn.train = p;
-      c->nn.train_S = S;
-      return TDKS_OK;
+  for (; !c->nn.train || S > c->nn.train_S; S /= 2) {
+    void* p = nullptr;
+    if (cudaMalloc(&p, nn_train_bytes(c->npts, S)) != cudaSuccess) {
+      cudaGetLastError();
+      if (S == 1) return fail(TDKS_ENOMEM, "training workspace");
+      continue;
     }
-    cudaGetLastError();
-    if (S == 1) return fail(TDKS_ENOMEM, "training workspace");
-    S /= 2;
+    if (c->nn.train && c->nn.train_S > 1) {
+      TDKS_CUDA(cudaStreamSynchronize(c->stream));
+      cudaFree(c->nn.train);
+    } else if (c->nn.train) {
+      c->allocs.push_back(c->nn.train);
+    }
+    c->nn.train = p;
+    c->nn.train_S = S;
+    return TDKS_OK;
   }
   return TDKS_OK;
 }
