@@ -306,7 +306,7 @@ def gpu_arm(args, rank, world, local_rank):
         J64.append(ctx64.read_step_observables()["J"])
     torch.cuda.synchronize()
     f64_sps = nref / (time.perf_counter() - tic)
-    st64 = ctx64.stats(reset=True)
+    st64, path64 = ctx64.stats(reset=True), ctx64.taylor_path()
     J64 = np.array(J64)
     ctx64.close()
     del u64
@@ -339,7 +339,8 @@ def gpu_arm(args, rank, world, local_rank):
                 c2.set_step_graph(False)
             ms, J, st = timed_steps(c2, u2, s, t0, args.warmup, args.steps, flush, record_j=True, label=name)
             o = c2.read_step_observables()
-            modes[name] = dict(ms=ms, J=J, st=st, fallbacks=o["fallbacks"], cell_scheme=c2.cell_variant())
+            modes[name] = dict(ms=ms, J=J, st=st, fallbacks=o["fallbacks"], cell_scheme=c2.cell_variant(),
+                               path=c2.taylor_path())
             c2.close()
     sweep = threshold_sweep(s, psi0, params, t0, args.warmup, args.steps, flush, J64, dev) if params is not None else None
     clk = clocks.stop()
@@ -368,6 +369,7 @@ def gpu_arm(args, rank, world, local_rank):
                           "J and norms of the input state fused into the first stage)",
                 "avg_launch_ms": k_ms, "launches_timed": st["calls"]["stencil_kernel"],
                 "buffer_scheme": cell_scheme(head["cell_scheme"] if head else None),
+                "taylor_path": taylor_path_name(head["path"]) if head else None,
                 "flops_per_launch": flops,
                 "peak_note": "measured FP32 FMA rate of this GPU (tdks_probe_fp32, FMA chains on every SM); "
                              f"derived {n_sm} SM x 128 lanes x 2 flop x max SM clock = {fp32_derived:.1f} TFLOP/s",
@@ -383,12 +385,16 @@ def gpu_arm(args, rank, world, local_rank):
                             "fallbacks": m["fallbacks"], "steps": args.warmup + args.steps,
                             "phase_ms_per_step": m["st"]["phase_ms"]}
     predictors["f64_pc_steps_per_s_host_synced"] = f64_sps
-    # the FP64 path is bound by the FP64 pipes: its cell kernel against the measured FP64 FMA rate
+    # the FP64 path: its Taylor launch against the measured FP64 FMA rate where the FP64 kernel runs; in fixed point
+    # (integer instructions) the same quotient is no share of a pipe, and is given under its own name
     k64 = st64["ms"]["stencil_kernel"] / max(1, st64["calls"]["stencil_kernel"])
     fp64_peak = T.probe_fp64()
-    predictors["f64_cell_kernel"] = {"avg_launch_ms": k64, "achieved_tflops": flops / (k64 * 1e-3) / 1e12,
+    r64 = flops / (k64 * 1e-3) / 1e12 / fp64_peak
+    fixed64 = path64 == T.PATH_FIXED
+    predictors["f64_cell_kernel"] = {"avg_launch_ms": k64, "path": taylor_path_name(path64),
+                                     "counted_tflops": flops / (k64 * 1e-3) / 1e12,
                                      "peak_tflops": fp64_peak, "peak_note": "measured FP64 FMA rate (tdks_probe_fp64)",
-                                     "frac": flops / (k64 * 1e-3) / 1e12 / fp64_peak}
+                                     "frac": None if fixed64 else r64, "counted_flops_over_fp64_rate": r64}
     if train_info:
         predictors["training"] = train_info
     if sweep:
@@ -648,8 +654,14 @@ def summary(line):
             "cubic_steps_per_s": best["cubic"]["steps_per_s"], "learned_fallbacks": best["learned"]["fallbacks"],
             "cubic_fallbacks": best["cubic"]["fallbacks"], "learned_J_rel_err": best["learned"]["J_rel_err_vs_f64_pc"],
             "cubic_J_rel_err": best["cubic"]["J_rel_err_vs_f64_pc"]}
-    out["f64_cell_kernel_frac_of_measured_fp64"] = g(pr, "f64_cell_kernel", "frac")
+    out["f64_taylor_launch_ms"] = g(pr, "f64_cell_kernel", "avg_launch_ms")
+    out["f64_taylor_counted_flops_over_fp64_rate"] = g(pr, "f64_cell_kernel", "counted_flops_over_fp64_rate")
     return out
+
+
+def taylor_path_name(path):
+    """The kernels of a context's Taylor launches (tdks_taylor_path)."""
+    return {1: "cell or tile kernels", 2: "slabs over a cluster", 3: "64-bit fixed point"}[path]
 
 
 def cell_scheme(v):
