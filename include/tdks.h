@@ -396,7 +396,8 @@ tdks_status tdks_nn_gradient(tdks_ctx* ctx, const double* vhist_dev, const doubl
  * Phases: 0 predictor Taylor kernel, 1 corrector Taylor kernel (and tdks_taylor_step),
  * 2 tdks_hpsi kernel, 3 Hartree + exchange (density-to-potential), 4 observables,
  * 5 everything else (potential combination, memsets), 6 the orbital stencil kernel launches alone
- * (the shared-memory cell kernel, or the tile stencil kernel of large grids), nested inside phases
+ * (the shared-memory cell kernel, the slab or fixed-point launches of tdks_taylor_path, or the tile
+ * stencil kernel of large grids), nested inside phases
  * 0-2 and also counted there.  With timing enabled the library records a CUDA event pair around
  * each phase on the context stream (a few microseconds of overhead per step).  `launches` counts
  * this library's kernel launches since the last reset, timing on or off. */

@@ -11,11 +11,15 @@
 //     5040 with centre -14350; D1: 672, -168, 32, -3 over 840), so the weighted sums are exact;
 //   * each axis sum is then multiplied once by a 57-bit coefficient dt/(2 h^2) ... as digits
 //     c = (ch 2^28 + cl) 2^-57: three multiply-adds into accumulators shared by all terms of the point.
-// A stage takes about 800 instructions per 32 points (multiply-adds at a quarter rate bound it) against
-// 7000 cycles for its 100 FP64 instructions.  One Taylor launch of 1024 orbitals of 20^3: 7.40 ms in FP64,
-// 1.48 ms here; of 8 orbitals of 16^3: 500 us and 47 us.  Error of one step against 113-bit arithmetic,
-// 20^3 and 16^3: 5.3e-17 and 5.9e-17 relative (the rounding of the result to FP64); the FP64 kernel 1.0e-16
-// and 6.2e-17.
+// A stage takes about 800 instructions per 32 points (multiply-adds at a quarter rate bound it: 64 % of the heavy FMA
+// pipe) against 7000 cycles for its 100 FP64 instructions.  One Taylor step of 1024 orbitals of 20^3: 7.00 ms in
+// FP64, 1.48 here (the launch 1.47, with the orbital written, the density and the current 1.85); of 8 orbitals of 16^3:
+// 500 us and 48 (the launch 36, and 51).  Error of one step against 113-bit arithmetic, l2 over an orbital, 20^3 and
+// 16^3: 5.3e-17 and 5.9e-17 relative (the rounding of the result to FP64); the FP64 kernel 1.0e-16 and 6.2e-17; the
+// largest error at any point is also the smaller of the two on seven grids.  The unit is one for a whole orbital, so
+// that single values below 2^-6 of the largest are less exact than in FP64, by 2^6 at the limit of kFxRange.  The density
+// is right to FP64 rounding of the values at every point; the current is 9e-18 of the density off on average (36 steps of
+// six cells), the FP64 kernel's 1.1e-17.
 //
 // An orbital is spread over a cluster of 1, 2, 4 or 8 CTAs, each owning a slab of planes in three
 // shared-memory copies (psi and two Horner vectors); the four planes above and below a slab are read from

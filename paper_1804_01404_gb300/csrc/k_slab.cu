@@ -14,13 +14,14 @@
 // All four Horner stages run in one launch; a stage takes two cluster barriers: after the local pass
 // (with the partial projections, which every CTA sends to every other) and after the nonlocal scatter.
 //
-// Taylor launch (with the projections) in a chain, microseconds, before -> here: 32^3 isolated, 16 orbitals,
-// 8 atoms 94 -> 55 (12 tile launches with a third of the SMs; now bound by the barriers and the latency of a
-// stage); 24^3 periodic, 1024 orbitals 866 -> 642 (its second copy no longer passes through scratch; bound by
-// shared-memory loads and issue slots); 12^3, 1024 orbitals 107 -> 84; 32 x 28 x 28, 128 orbitals, 3 atoms
-// 204 -> 154 (with the projectors' values in shared memory one CTA fits an SM instead of two: 204).  Not
-// faster: 15 x 18 x 21, 324 orbitals, 4 atoms (125 either way: their waves over 152 SMs).  No rule on sizes tells these apart, so a context
-// times one launch of each and keeps the faster (tune_cell, tune_tile).
+// Taylor steps (with the projections, no density) in a chain, microseconds, without -> here: 32^3 isolated, 16 orbitals,
+// 8 atoms 90 -> 55 (12 tile launches with a third of the SMs; now bound by the barriers and the latency of a
+// stage); 24^3 periodic, 1024 orbitals, 3 atoms 709 -> 621 (its second copy no longer passes through scratch; bound by
+// shared-memory loads and issue slots); 12^3, 1024 orbitals, 1 atom 103 -> 90; 32 x 28 x 28, 128 orbitals, 3 atoms
+// 204 -> 156 (with the projectors' values in shared memory one CTA fits an SM instead of two: 204).  Not
+// faster: 15 x 18 x 21, 324 orbitals, 4 atoms (125 -> 156: odd rows are read point by point), 20^3 with its size built in
+// (217 -> 353).  No rule on sizes tells these apart, so a context times one launch of each and keeps the faster
+// (tune_cell, tune_tile).
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -1024,7 +1024,7 @@ tdks_status tune_cell(tdks_ctx* c) {
   c->cell_ms[0] = c->cell_ms[1] = c->cell_ms[2] = c->cell_ms[3] = -1.f;
   const bool schemes = cell_ip_ok(c) || cell_geom_ok(c);
   // the slab launch, against scheme 0 alone once each after one untimed launch; with the grid size built in only where
-  // few orbitals leave SMs idle (1024 of 20^3: 430 us in slabs, 217 with the size built in)
+  // few orbitals leave SMs idle (1024 of 20^3: 353 us in slabs, 217 with the size built in)
   const bool slab = c->slab_ok && !(cell_geom_ok(c) && is_f32(c) && c->ncell * c->nk * c->norb >= 304);
   if (c->tiled || (!schemes && !slab)) return TDKS_OK;
   const int reps = schemes ? 2 : 1;
