@@ -43,6 +43,7 @@ struct FxArgs {
   int write_out;
   double* obs;              // nullable: per orbital {norm, J_loc[3], J_nl[3], 0}
   int* need;                // [norb_tot] 1: out of the fixed-point range, nothing written
+  int* vbad;                // [ncell] 1: a potential value beyond the digits (cleared by the FP64 kernel launched after)
 };
 
 // How a grid is split for `norb_tot` orbitals; false: one CTA of a cluster of 8 cannot hold its slab.

@@ -44,7 +44,6 @@ namespace tdks {
 namespace {
 
 constexpr int kFxThreads = 512;
-constexpr int kVBad = 0x7fffffff;      // digit of a potential outside the coefficient range
 constexpr int kFxStaticReserve = 4 * 1024;
 // Orbitals with a block of 4 x 4 x 4 points all 2^12 below their largest value go to the FP64 kernel: they decay
 // into a vacuum, where an FP64 stencil is right to 2^-53 of its own neighbours and a unit here is 2^-59 of the
@@ -229,7 +228,8 @@ struct ObsAcc {
 
 }  // namespace
 
-// Potential digits dt V (kVBad outside |dt V| < 1), phase factors exp(i q.d) of every (cell, k) and
+// Potential digits dt V (|dt V| < 1; a value outside flags its cell, whose orbitals then return before their first
+// stage), phase factors exp(i q.d) of every (cell, k) and
 // sphere entry: q = k + A' of the step (ph) and of its observables (pho, nullable).  One launch before
 // the orbitals: 7 us of sincos for 64 k and 1018 entries, which each of the norb orbitals of a k would
 // otherwise repeat (32 k cycles each).
@@ -240,7 +240,9 @@ __global__ void __launch_bounds__(128) k_fx_prep(FxArgs a) {
   for (ll i = (ll)blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += (ll)gridDim.x * blockDim.x) {
     if (i < nv) {
       const double v = a.V64[i] * a.dt;
-      a.V[i] = fabs(v) < 1.0 ? digits28(__double2ll_rn(v * 144115188075855872.0)) : make_int2(kVBad, 0);
+      const bool in = fabs(v) < 1.0;
+      a.V[i] = in ? digits28(__double2ll_rn(v * 144115188075855872.0)) : make_int2(0, 0);
+      if (!in) a.vbad[a.vstride ? i / a.npts : 0] = 1;
       continue;
     }
     ll j = i - nv;
@@ -420,7 +422,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_cell_fx(FxArgs a) {
     }
     const double dg = (a.diag + 0.5 * q2) * a.dt;
     bound += fabs(dg);
-    s_cbad = !(bound < 4.1) || fabs(dg) >= 3.0;     // (with |dt V| < 1 a digit holds the sum)
+    s_cbad = !(bound < 4.1) || fabs(dg) >= 3.0 || a.vbad[a.vstride ? cell : 0];   // (with |dt V| < 1 a digit holds the sum)
     s_diag = digits28(s_cbad ? 0 : __double2ll_rn(dg * 144115188075855872.0));
     if (OBS) {
       const double* Ao = a.Ap_obs_cell ? a.Ap_obs_cell + 3 * cell : a.Ap_obs;
@@ -578,7 +580,6 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_cell_fx(FxArgs a) {
               if (ACC) oa.cur(ax, ux, uy, d);
             }
           }
-          bad |= vd.x == kVBad;
           const int2 dg = make_int2(vd.x + s_diag.x, vd.y + s_diag.y);
           tx.add(u.x, u.y, dg);
           ty.add(u.z, u.w, dg);

@@ -990,8 +990,11 @@ __global__ void __launch_bounds__(kMaxThreads<T, IP, GEOM>(), kMinBlocks<T, IP, 
   T* tbeta = reinterpret_cast<T*>(smem_raw + geom_table_offset<T>(a.nx, a.ny, a.nz, ps, a.nsph, a.natom, IP));
   int* tidx = reinterpret_cast<int*>(tbeta + 4 * (size_t)a.nsph);
   const int orb = blockIdx.x;
-  if (a.need && a.need[orb] == 0) return;          // already propagated in fixed point (k_fixed.cu)
   const int cell = orb / (a.nk * a.norb);
+  if (a.need) {
+    if (threadIdx.x == 0 && orb == cell * a.nk * a.norb) a.vbad[cell] = 0;
+    if (a.need[orb] == 0) return;                  // already propagated in fixed point (k_fixed.cu)
+  }
   const int k = (orb - cell * a.nk * a.norb) / a.norb;
   const C* psi = a.psi_in + (size_t)orb * a.npts;
   C* gnxt = DBUF ? nullptr : scratch + (size_t)orb * a.npts;

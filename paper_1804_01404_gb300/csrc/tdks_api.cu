@@ -110,7 +110,7 @@ struct tdks_ctx {
   int4 *d_fx_beta = nullptr, *d_fx_ph = nullptr;
   int2 *d_fx_d = nullptr, *d_fx_rng = nullptr, *d_fx_sp = nullptr, *d_fx_V = nullptr;
   double* d_fx_fac = nullptr;    // [2][natom][4]: ecfac / dt, jfac
-  int* d_fx_need = nullptr;
+  int *d_fx_need = nullptr, *d_fx_vbad = nullptr;
   float* d_kwsplit = nullptr;    // [nk][2]: each k weight as a float pair (the density fold)
   // grid arrays
   double *d_vloc = nullptr, *d_vhxc = nullptr, *d_vpred = nullptr, *d_rho = nullptr,
@@ -640,8 +640,10 @@ tdks_status fx_setup(tdks_ctx* c, const ProjectorTables& T) {
         no_room(upload(c, &c->d_fx_fac, fac)) || no_room(dalloc(c, &c->d_fx_ph, 2 * (size_t)c->ncell * c->nk * c->nsph)))
       return TDKS_OK;
   }
-  if (no_room(dalloc(c, &c->d_fx_V, (size_t)c->npts * c->ncell)) || no_room(dalloc(c, &c->d_fx_need, (size_t)tot)))
+  if (no_room(dalloc(c, &c->d_fx_V, (size_t)c->npts * c->ncell)) || no_room(dalloc(c, &c->d_fx_need, (size_t)tot)) ||
+      no_room(dalloc(c, &c->d_fx_vbad, (size_t)c->ncell)))
     return TDKS_OK;
+  TDKS_CUDA(cudaMemsetAsync(c->d_fx_vbad, 0, sizeof(int) * (size_t)c->ncell, c->stream));
   c->fx_ok = true;
   return TDKS_OK;
 }
@@ -681,7 +683,7 @@ FxArgs make_fx_args(const tdks_ctx* c, const OrbArgs<double>& o) {
   a.ph = c->d_fx_ph;
   a.pho = c->d_fx_ph ? c->d_fx_ph + (size_t)c->ncell * c->nk * c->nsph : nullptr;
   a.phstride = o.Ap_cell || o.Ap_obs_cell ? (long long)c->nk * c->nsph : 0;
-  a.rho = o.rho; a.write_out = o.write_out; a.obs = o.obs; a.need = c->d_fx_need;
+  a.rho = o.rho; a.write_out = o.write_out; a.obs = o.obs; a.need = c->d_fx_need; a.vbad = c->d_fx_vbad;
   return a;
 }
 
@@ -751,6 +753,7 @@ tdks_status orbital_kernel(tdks_ctx* c, int mode, const void* in, void* out, con
       if (mode == 1 && fx_use(c, dt)) {           // the FP64 kernel then takes the orbitals out of range
         TDKS_CUDA(launch_cell_fx(make_fx_args(c, a), c->grid.periodic != 0, obs_start, c->stream));
         a.need = c->d_fx_need;
+        a.vbad = c->d_fx_vbad;
         c->launches += 2;
       }
       TDKS_CUDA(launch_smem_orbital<double>(a, mode, static_cast<double2*>(c->d_scratch), c->stream));

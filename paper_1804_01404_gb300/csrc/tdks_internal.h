@@ -105,6 +105,7 @@ struct OrbArgs {
   double* obs;              // nullable: per-orbital {norm, jloc[3], jnl[3], 0}
   int obs_at_start;         // 1: observables of the input orbital (first stage), 0: of the output
   const int* need;          // nullable: [norb_tot] orbitals to work on (1) or to leave (0)
+  int* vbad;                // with need: [ncell] flags that the first orbital's CTA of a cell clears
   C* backup;                // nullable: copy of the input orbitals, written while they are loaded
   // batches of cells (multiscale): orbitals are [ncell][nk][norb], potentials [ncell][npts]
   int ncell;                // cells in the batch (1 for a single system)

@@ -133,3 +133,43 @@ def test_current_no_further_off_than_fp64(n, natom):
                     ref *= -2 * ld(s.dV) / ld(s.dV * s.npts)
                     err[scheme].append(float(abs(J[a] - ref) / (norm / s.npts)))
     assert np.mean(err[None]) <= np.mean(err[0]), (np.mean(err[None]), np.mean(err[0]))
+
+
+def test_potential_beyond_its_digits():
+    """A well of |dt V| > 1: every orbital through the FP64 kernel, bit for bit; in a batch only the cell that has it
+    (and the next step, with the well gone by a smaller dt, in fixed point again)."""
+    n, h = (12, 10, 9), (0.5,) * 3
+    s = box(n, h, True, 3, [W.Atom((2.0, 2.5, 2.0), 60.0)], W.Projectors(r_cut=1.5))
+    u0 = torch.from_numpy(W.initial_orbitals(s, 1)).cuda()
+    ctx = tdks.Context(s, precision="f64", hartree=False, xc=False)
+    assert float(ctx.grid_array(0).abs().max()) * 0.02 > 1.0
+    got = {}
+    for path in (tdks.PATH_FIXED, tdks.PATH_KERNELS):
+        ctx.taylor_path(path)
+        for dt in (0.02, 0.002, -0.02):
+            u = u0.clone()
+            ctx.update_potential(u)
+            ctx.taylor_step(u, dt, [0.1, 0.2, -0.1])
+            got[path, dt] = u
+    for dt in (0.02, -0.02):
+        assert torch.equal(got[tdks.PATH_FIXED, dt], got[tdks.PATH_KERNELS, dt])
+    a, b = got[tdks.PATH_FIXED, 0.002], got[tdks.PATH_KERNELS, 0.002]
+    assert not torch.equal(a, b) and float((a - b).norm() / b.norm()) < 2e-15
+
+
+def test_one_cell_of_a_batch_beyond():
+    """Cells of a batch whose densities differ: the Hartree potential of one exceeds the digits, the others' do not."""
+    s = box((10, 9, 8), (0.5, 0.55, 0.6), True, 2)
+    ctx = tdks.Context(s, precision="f64", ncell=3)
+    u0 = torch.from_numpy(np.stack([W.initial_orbitals(s, i) for i in range(3)])).cuda()
+    u0[1] *= 60.0                                        # 3600 times the electrons
+    ctx.update_potential(u0)
+    out = []
+    for path in (tdks.PATH_FIXED, tdks.PATH_KERNELS):
+        ctx.taylor_path(path)
+        u = u0.clone()
+        ctx.taylor_step(u, 0.02)
+        out.append(u)
+    assert torch.equal(out[0][1], out[1][1])
+    for i in (0, 2):
+        assert not torch.equal(out[0][i], out[1][i]) and float((out[0][i] - out[1][i]).norm() / out[1][i].norm()) < 2e-15
