@@ -482,7 +482,8 @@ tdks_status tdks_cell_variant(tdks_ctx* ctx, int set, int* variant, float* tune_
  * value a unit, over one to eight SMs.  Orbitals that do not fit that -- not finite, beyond 2^+-423,
  * 2^12 below their largest value in whole blocks of 4 x 4 x 4 points, a time step or a wave vector
  * beyond the coefficients -- are propagated by the cell kernels, in the same call.
- * At tdks_init FP64 cell contexts that can take TDKS_PATH_FIXED do; FP32 contexts that can take
+ * At tdks_init FP64 cell contexts that can take TDKS_PATH_FIXED do, but for the smallest grids (periodic below
+ * 112 points, isolated below 160), which leave its CTAs' threads idle; FP32 contexts that can take
  * TDKS_PATH_SLAB time one launch of it (tiled contexts: a Taylor step of up to 304 orbitals) against the
  * other kernels and keep the faster; cells of a built-in size (schemes 2 and 3) with 304 orbitals or more
  * keep those.  The trial runs are most of tdks_init: 3 to 7 ms in FP32, 54 ms for 1024 FP64 orbitals of

@@ -382,6 +382,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_cell_fx(FxArgs a) {
   const int2 third = digits28(48038396025285291LL);
 
   // the slab as FP64 into the first copy, its largest exponent, a copy for a fallback (predicted steps)
+  const int vbad = tid == 0 ? a.vbad[a.vstride ? cell : 0] : 0;
   unsigned mx = 0;
   const int nown = (zend - zbeg) * nxy;
   double2* raw = reinterpret_cast<double2*>(buf);
@@ -422,7 +423,7 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_cell_fx(FxArgs a) {
     }
     const double dg = (a.diag + 0.5 * q2) * a.dt;
     bound += fabs(dg);
-    s_cbad = !(bound < 4.1) || fabs(dg) >= 3.0 || a.vbad[a.vstride ? cell : 0];   // (with |dt V| < 1 a digit holds the sum)
+    s_cbad = !(bound < 4.1) || fabs(dg) >= 3.0 || vbad;   // (with |dt V| < 1 a digit holds the sum)
     s_diag = digits28(s_cbad ? 0 : __double2ll_rn(dg * 144115188075855872.0));
     if (OBS) {
       const double* Ao = a.Ap_obs_cell ? a.Ap_obs_cell + 3 * cell : a.Ap_obs;

@@ -105,6 +105,7 @@ struct tdks_ctx {
   // fixed-point Taylor launches of FP64 orbitals (k_fixed.cu): split of an orbital over a cluster, digit
   // tables of the projectors, digits of the step potential and of the phases, per-orbital range flags
   bool fx_ok = false;            // the grid, the projectors and the options allow it
+  bool fx_on = false;            // ... and it is the faster path
   int fx_ncta = 1, fx_zl = 0, fx_zlen = 0, fx_nseg = 0, fx_sN = 0, fx_Kb = 0;
   double fx_nl_bound = 0.0;      // largest row sum of |V_NL| and of |E_p dV beta|
   int4 *d_fx_beta = nullptr, *d_fx_ph = nullptr;
@@ -645,6 +646,10 @@ tdks_status fx_setup(tdks_ctx* c, const ProjectorTables& T) {
     return TDKS_OK;
   TDKS_CUDA(cudaMemsetAsync(c->d_fx_vbad, 0, sizeof(int) * (size_t)c->ncell, c->stream));
   c->fx_ok = true;
+  // Grids with fewer points than a CTA's columns leave most of its 512 threads idle, where several FP64 CTAs share an SM.
+  // A Taylor step of 160 and 2000 orbitals, FP64 / fixed point in us: isolated 4^3 21/33 and 77/127, 5^3 29/33 and 149/138,
+  // 6^3 41/37 and 246/164; steps of periodic cells 4^3 125/150 and 387/596, 4 x 4 x 8 165/156 and 668/602.
+  c->fx_on = c->npts >= (c->grid.periodic ? 112 : 160);
   return TDKS_OK;
 }
 
@@ -687,10 +692,12 @@ FxArgs make_fx_args(const tdks_ctx* c, const OrbArgs<double>& o) {
   return a;
 }
 
+bool fx_path(const tdks_ctx* c) { return c->path == TDKS_PATH_AUTO ? c->fx_on : c->fx_ok && c->path == TDKS_PATH_FIXED; }
+
 // Whether a Taylor launch of step dt runs in fixed point: the weights of the step stay in the range of
 // its coefficients (the kernel checks the wave vector, the potential and the orbital themselves).
 bool fx_use(const tdks_ctx* c, double dt) {
-  if (!c->fx_ok || c->path == TDKS_PATH_KERNELS || !std::isfinite(dt)) return false;
+  if (!fx_path(c) || !std::isfinite(dt)) return false;
   double s = 0.0;
   for (int d = 0; d < 3; ++d) s += (3.251 + 1.4237) / (c->grid.h[d] * c->grid.h[d]);
   return std::fabs(dt) * s < 4.0 && std::fabs(dt) * c->fx_nl_bound < 0.9;
@@ -699,7 +706,7 @@ bool fx_use(const tdks_ctx* c, double dt) {
 // the path of the Taylor launches (of a usual step)
 int taylor_path(const tdks_ctx* c) {
   if (slab_use(c)) return TDKS_PATH_SLAB;
-  return c->fx_ok && c->path != TDKS_PATH_KERNELS ? TDKS_PATH_FIXED : TDKS_PATH_KERNELS;
+  return fx_path(c) ? TDKS_PATH_FIXED : TDKS_PATH_KERNELS;
 }
 
 // phase: profiling phase (-1: H u -> hpsi, a written Taylor result -> corrector, else predictor)

@@ -81,6 +81,26 @@ def test_paths_of_contexts():
         ctx.close()
 
 
+def test_smallest_fp64_grids():
+    """Grids that fill less than a CTA keep the FP64 kernel, and can be put on the fixed-point path."""
+    for n, periodic, want in (((4, 4, 4), True, KERNELS), ((4, 4, 8), True, FIXED), ((5, 5, 5), False, KERNELS),
+                              ((6, 6, 6), False, FIXED)):
+        s = system(n, (0.6,) * 3, periodic, 3, 0, 1)
+        ctx = tdks.Context(s, precision="f64")
+        assert ctx.taylor_path() == want
+        u0 = orbitals(s).to(torch.complex128)
+        out = []
+        for path in (KERNELS, FIXED, tdks.PATH_AUTO):
+            ctx.taylor_path(path)
+            u = u0.clone()
+            ctx.update_potential(u)
+            ctx.taylor_step(u, 0.02)
+            out.append(u)
+        assert rel(out[1], out[0]) < 2e-15                   # (as in test_gpu_fixed.py)
+        assert torch.equal(out[2], out[want == FIXED])
+        ctx.close()
+
+
 def test_graph_of_predicted_steps_follows_the_path():
     s = system((14, 15, 16), (0.5, 0.45, 0.4), True, 7, 2, 3)
     u0 = orbitals(s)
