@@ -355,7 +355,7 @@ template <bool PER, int OBS, bool ISO, int ZL>
 __global__ void __launch_bounds__(kFxThreads, 1) k_cell_fx(FxArgs a) {
   extern __shared__ __align__(16) unsigned char fx_smem[];
   __shared__ unsigned s_max[8], s_min[8], s_flag[8];
-  __shared__ unsigned s_wmax[kFxThreads / 32], s_wmin[kFxThreads / 32];
+  __shared__ unsigned s_wmax[kFxThreads / 32];
   __shared__ int2 s_cd[3], s_diag;
   __shared__ int s_cbad;
   __shared__ double s_qo[3], s_jnl[3], s_obs[8][4];
@@ -442,12 +442,14 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_cell_fx(FxArgs a) {
     paddr[i] = ad;
   }
   __syncthreads();
-  // the smallest largest value of a block: four rows of four planes (of the slab; the last rows and planes where they
-  // do not divide by four) and a group of each row, the group of its x-th point
-  unsigned mn = 0x7fffffffu;
-  {
+  if (ncta > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (warp == 0) {
+    // the smallest largest value of a block: four rows of four planes (of the slab; the last rows and planes where they
+    // do not divide by four) and a group of each row, the group of its x-th point
+    unsigned mn = 0x7fffffffu;
     const int nbx = a.nx % 4 == 0 ? a.nx / 4 : (a.nx + 2) / 4 + 1, nby = (a.ny + 3) / 4, nzl = zend - zbeg;
-    for (int b = tid; b < nbx * nby * ((nzl + 3) / 4); b += blockDim.x) {
+#pragma unroll 2
+    for (int b = lane; b < nbx * nby * ((nzl + 3) / 4); b += 32) {
       const int r = b / nbx, bz = r / nby, x = min(4 * (b - r * nbx), a.nx - 1);
       const int y0 = min(4 * (r - bz * nby), a.ny - 4), z0 = max(min(4 * bz, nzl - 4), 0);
       unsigned m = 0;
@@ -455,26 +457,21 @@ __global__ void __launch_bounds__(kFxThreads, 1) k_cell_fx(FxArgs a) {
       for (int j = 0; j < 16; ++j) m = max(m, grp[(min(z0 + (j >> 2), nzl - 1) * nxy + (y0 + (j & 3)) * a.nx + x) >> 2]);
       mn = min(mn, m);
     }
-  }
-  mn = __reduce_min_sync(0xffffffffu, mn);
-  if (lane == 0) s_wmin[warp] = mn;
-  __syncthreads();
-  if (ncta > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-  if (warp == 0) {
-    unsigned w = lane < (int)(blockDim.x >> 5) ? s_wmax[lane] : 0u, v = lane < (int)(blockDim.x >> 5) ? s_wmin[lane] : 0x7fffffffu;
+    unsigned w = lane < (int)(blockDim.x >> 5) ? s_wmax[lane] : 0u;
     w = __reduce_max_sync(0xffffffffu, w);
-    v = __reduce_min_sync(0xffffffffu, v);
+    mn = __reduce_min_sync(0xffffffffu, mn);
     if (lane < ncta) {
       if (ncta > 1) {
         st_cluster32(map_cta(smem_addr(&s_max[rank]), lane), w);
-        st_cluster32(map_cta(smem_addr(&s_min[rank]), lane), v);
+        st_cluster32(map_cta(smem_addr(&s_min[rank]), lane), mn);
       } else {
         s_max[0] = w;
-        s_min[0] = v;
+        s_min[0] = mn;
       }
     }
   }
   if (ncta > 1) cluster_sync(); else __syncthreads();
+  unsigned mn = 0x7fffffffu;
   mx = 0;
   for (int r = 0; r < ncta; ++r) {
     mx = max(mx, s_max[r]);
