@@ -486,7 +486,7 @@ tdks_status tdks_cell_variant(tdks_ctx* ctx, int set, int* variant, float* tune_
  * 112 points, isolated below 160), which leave its CTAs' threads idle; FP32 contexts that can take
  * TDKS_PATH_SLAB time one launch of it (tiled contexts: a Taylor step of up to 304 orbitals) against the
  * other kernels and keep the faster; cells of a built-in size (schemes 2 and 3) with 304 orbitals or more
- * keep those.  The trial runs are most of tdks_init: 3 to 7 ms in FP32, 54 ms for 1024 FP64 orbitals of
+ * keep those.  The trial runs are most of tdks_init: 3 to 7 ms in FP32, 17 ms for 1024 FP64 orbitals of
  * 20^3.
  *   set   : -1 leaves the path as it is; TDKS_PATH_AUTO goes back to the choice of tdks_init (the
  *           scheme of tdks_cell_variant stays as it was set); the others force that path.

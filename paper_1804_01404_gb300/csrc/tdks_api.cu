@@ -1038,10 +1038,13 @@ tdks_status tune_cell(tdks_ctx* c) {
   const bool slab = c->slab_ok && !(cell_geom_ok(c) && is_f32(c) && c->ncell * c->nk * c->norb >= 304);
   if (c->tiled || (!schemes && !slab)) return TDKS_OK;
   const int reps = schemes ? 2 : 1;
-  // at most 1216 orbitals, fewer where the device has no room for a copy of them; with room for none scheme 0 stays
+  // at most 1216 orbitals (304 of FP64 contexts whose launches run in fixed point, where the schemes only take what that
+  // leaves: 54 -> 17 ms of tdks_init for 1024 of 20^3), fewer where the device has no room for a copy of them; with room
+  // for none scheme 0 stays
   const size_t csz = is_f32(c) ? sizeof(float2) : sizeof(double2);
-  int tnk = std::min(c->nk, 1216), tnorb = std::min(c->norb, 1216 / tnk);
-  int tcell = tnk == c->nk && tnorb == c->norb ? std::min(c->ncell, 1216 / (tnk * tnorb)) : 1;
+  const int most = c->fx_on ? 304 : 1216;
+  int tnk = std::min(c->nk, most), tnorb = std::min(c->norb, most / tnk);
+  int tcell = tnk == c->nk && tnorb == c->norb ? std::min(c->ncell, most / (tnk * tnorb)) : 1;
   void* buf = nullptr;
   while (cudaMalloc(&buf, csz * (size_t)tcell * tnk * tnorb * c->npts) != cudaSuccess) {
     cudaGetLastError();
